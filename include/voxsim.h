@@ -181,7 +181,8 @@ const char* sim_last_error(const voxsim_ctx* ctx);
  * component labelling hit its iteration bound) give SIM_ETIMEOUT, words[0] bit 1 (a material
  * id out of range in device-memory genomes) SIM_EINVAL, none SIM_OK.  words[2] bit 3 is the
  * stepping's (a segment of the lattice step gave up its bounded wait for its robots' previous
- * segment, see sim_step_n), reported as SIM_ETIMEOUT by sim_fitness into host memory.
+ * segment, see sim_step_n, or a warp of the lattice step or the adjoint its wait for a
+ * neighbouring warp's data), reported as SIM_ETIMEOUT by sim_fitness into host memory.
  * words: host int32 [4].
  * Needs no device: it lets a caller (and the test-suite) check the mapping without making a
  * device-side wait run out.  The paper has no counterpart.  Errors: SIM_EINVAL for NULL. */

@@ -27,6 +27,8 @@
 #include "common.cuh"
 #include "physics.cuh"
 #include "tmem.cuh"
+#include "shared_rows.cuh"
+#include "warp_flow.cuh"
 
 namespace vx {
 namespace {
@@ -70,14 +72,14 @@ __device__ __forceinline__ void cells_load(uint32_t tm, uint32_t (&v)[6])
 // transpose and one 4-column store of the updated sums after it.  Held in registers next to the
 // sweep's other state they spilled to local memory, which misses L1 beside 221 KB of shared
 // memory: 1.5x the time of this version.
-// CUBE8: every item is one 8 x 8 x 8 robot in a 768-thread slot; strides and plane stride are
-// compile-time constants (immediate shared-memory offsets), as in the forward kernel.
-template <bool CUBE8>
+// GRID8: as in the forward kernel.
+template <bool GRID8>
 __global__ void __launch_bounds__(kBlock, 1) k_adjoint_lattice(AdjointArgs a)
 {
-    extern __shared__ __align__(16) float4 sm4[];
     __shared__ int sh_item[4];
     __shared__ uint32_t sh_tmem;
+    __shared__ FlowBars sh_flow;
+    float4* const sm4 = reinterpret_cast<float4*>(lattice_smem);
     const int tid = threadIdx.x, warp = tid >> 5;
     if (warp == 0) tmem_alloc_warp(&sh_tmem);
     tmem_fence_before();
@@ -85,6 +87,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_adjoint_lattice(AdjointArgs a)
     tmem_fence_after();
     const uint32_t tm = tmem_warp_base(sh_tmem, warp);
     const StepConst c = a.c;
+    flow_create(sh_flow);
     for (;;) {
         if (tid == 0) {
             const int it = atomicAdd(a.queue, 1);
@@ -98,19 +101,24 @@ __global__ void __launch_bounds__(kBlock, 1) k_adjoint_lattice(AdjointArgs a)
         __syncthreads();
         if (!sh_item[3]) break;
         const int first = sh_item[0], count = sh_item[1], gthreads = sh_item[2];
-        const int group = CUBE8 ? 0 : tid / gthreads, lt = CUBE8 ? tid : tid % gthreads;
+        const int group = GRID8 ? 0 : tid / gthreads, lt = GRID8 ? tid : tid % gthreads;
         __syncthreads();
         if (group < count) {                              // whole warps (slots are multiples of 32)
             const int r = a.item_robots[first + group];
             const int nx = a.pv.dims[3 * r], ny = a.pv.dims[3 * r + 1], nz = a.pv.dims[3 * r + 2];
-            const int X = CUBE8 ? 9 : nx + 1, XY = CUBE8 ? 81 : (nx + 1) * (ny + 1), C = CUBE8 ? 729 : XY * (nz + 1);
+            const int X = nx + 1, XY = X * (ny + 1), C = XY * (nz + 1);
+            // row strides in shared memory: the grid's own, or those of 9 x 9 x 9 corners
+            const int RX = GRID8 ? 9 : X, RXY = GRID8 ? 81 : XY;
             const int64_t mo = a.pv.moff[r];
             const int bar = 1 + group;
-            const int S = CUBE8 ? kBlock : gthreads;
-            float4* su = sm4 + (size_t)group * kLatticeSlotVec4 * S;
+            const int S = GRID8 ? kBlock : gthreads;
+            // u, adjoint force and 13 far-end shares per corner
+            float4* su = sm4 + (size_t)group * kSlotVec4 * S;
             float4* sg = su + S;
             float4* sl = sg + S;
+            const NarrowRows nu(0, kBlock), ng(12 * kBlock, kBlock), nl(24 * kBlock, 13 * kBlock);   // GRID8
             const int cidx = lt;
+            const int row = GRID8 ? cidx + (cidx / X) * (9 - X) + (cidx / XY) * (81 - 9 * (ny + 1)) : cidx;
             const bool in = cidx < C;
             // warps past the robot's corners skip the transposes (a uniform branch, so the
             // warp-collective tensor-memory accesses stay converged)
@@ -147,7 +155,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_adjoint_lattice(AdjointArgs a)
                 tmem_wait_st();
             }
             const float z0 = in ? a.u0[o].w : 0.f;
-            float4* stage_u = sm4 + (size_t)kLatticeSlotVec4 * kBlock;           // [2][kBlock]
+            float4* stage_u = reinterpret_cast<float4*>(sm4 + kSlotVec4 * kBlock);   // [2][kBlock]
             float2* stage_f = reinterpret_cast<float2*>(stage_u + 2 * kBlock);   // [2][kBlock]
             int sb = 0;
             if (in) {
@@ -156,17 +164,17 @@ __global__ void __launch_bounds__(kBlock, 1) k_adjoint_lattice(AdjointArgs a)
                 cp_async(&stage_f[tid], &a.rec_f[ro], 8);
             }
             cp_async_commit();
-            int Xs = X, XYs = XY, Ss = S;
-            for (int n = a.n1 - 1; n >= a.n0; --n) {
-                // the lattice offsets are recomputed every step rather than hoisted out of the
-                // loop and spilled: an opaque copy of the strides hides their invariance
-                if constexpr (!CUBE8) asm volatile("" : "+r"(Xs), "+r"(XYs), "+r"(Ss));
+            // phases of WarpFlow: A is the spring transposes, B the gather and the mass part
+            WarpFlow flow;
+            if (warp_in)
+                flow.init(sh_flow, GRID8 ? 0 : (group * gthreads) >> 5, lt >> 5, (C + 31) >> 5, XY + X + 1);
+            group_sync(bar, gthreads);
+            uint32_t ph = 0;
+            if (warp_in) for (int n = a.n1 - 1; n >= a.n0; --n, ph ^= 1u) {
                 // direction 0's cells, read while the mass part runs
                 uint32_t cur[6];
-                if (warp_in) {
-                    __syncwarp();                         // converged for the collective loads
-                    cells_load<0>(tm, cur);
-                }
+                __syncwarp();                             // converged for the collective loads
+                cells_load<0>(tm, cur);
                 cp_async_wait_all();
                 float4 un = make_float4(0.f, 0.f, 0.f, 0.f);
                 float2 fh = make_float2(0.f, 0.f);
@@ -184,48 +192,55 @@ __global__ void __launch_bounds__(kBlock, 1) k_adjoint_lattice(AdjointArgs a)
                 float lFx = 0.f, lFy = 0.f, lFz = 0.f;
                 if (mass) mass_adjoint(__float_as_uint(un.w), z0 + un.z, fh, lux, luy, luz, lvx, lvy, lvz, lFx, lFy, lFz, c);
                 if (in) {
-                    su[cidx] = un;
-                    sg[cidx] = make_float4(lFx, lFy, lFz, 0.f);
+                    if constexpr (GRID8) {
+                        nu.store(row, un.x, un.y, un.z);
+                        ng.store(row, lFx, lFy, lFz);
+                    } else {
+                        su[cidx] = un;
+                        sg[cidx] = make_float4(lFx, lFy, lFz, 0.f);
+                    }
                 }
-                group_sync(bar, gthreads);
+                flow.arrive_b();
                 const float2 sc = a.sc[n];
+                if (!flow.wait_b(ph)) { tmem_wait_ld6(cur); atomicOr(a.status, 8); break; }
                 // own forward springs: as in the register version, branch-free (an absent spring
                 // has k = 0 and the corner itself as far end); lanes past the corners compute on
                 // their own unused rows and their results are never read
-                if (warp_in) {
+                __syncwarp();
+                tmem_wait_ld6(cur);
+                for_each_dir([&](auto t) {
+                    constexpr int d = decltype(t)::value;
+                    if constexpr (d > 0) {
+                        cells_load<d>(tm, cur);
+                        tmem_wait_ld6(cur);
+                    }
+                    const bool has = (fl >> d) & 1u;
+                    const int nb = has ? row + lattice_offset<d>(RX, RXY) : row;
+                    const float4 ub = GRID8 ? nu.load(nb) : su[nb], gb = GRID8 ? ng.load(nb) : sg[nb];
+                    const float k = __uint_as_float(cur[0]);
+                    const SpringEval e = spring_eval_ends<d>(ub, un, c.edge,
+                        lattice_rest<d>(c), lattice_rest_sq<d>(c), k, __uint_as_float(cur[1]),
+                        __uint_as_float(cur[2]), sc.x, sc.y);
+                    float ldx, ldy, ldz, dk, da, db;
+                    // lambda_F_a - lambda_F_b, x and y as one paired fused multiply-add
+                    const float2 lf = __ffma2_rn(make_float2(gb.x, gb.y), kMinusOne2, make_float2(lFx, lFy));
+                    spring_adjoint(e, k, lf.x, lf.y, lFz - gb.z, sc.x, sc.y, ldx, ldy, ldz, dk, da, db);
+                    lux -= ldx; luy -= ldy; luz -= ldz;
+                    if constexpr (GRID8) nl.store(13 * row + d, ldx, ldy, ldz);
+                    else sl[13 * cidx + d] = make_float4(ldx, ldy, ldz, e.ext);
                     __syncwarp();
-                    tmem_wait_ld6(cur);
-                    for_each_dir([&](auto t) {
-                        constexpr int d = decltype(t)::value;
-                        if constexpr (d > 0) {
-                            cells_load<d>(tm, cur);
-                            tmem_wait_ld6(cur);
-                        }
-                        const bool has = (fl >> d) & 1u;
-                        const int nb = has ? cidx + lattice_offset<d>(Xs, XYs) : cidx;
-                        const float4 ub = su[nb], gb = sg[nb];
-                        const float k = __uint_as_float(cur[0]);
-                        const SpringEval e = spring_eval_ends<d>(ub, un, c.edge,
-                            lattice_rest<d>(c), lattice_rest_sq<d>(c), k, __uint_as_float(cur[1]),
-                            __uint_as_float(cur[2]), sc.x, sc.y);
-                        float ldx, ldy, ldz, dk, da, db;
-                        // lambda_F_a - lambda_F_b, x and y as one paired fused multiply-add
-                        const float2 lf = __ffma2_rn(make_float2(gb.x, gb.y), kMinusOne2, make_float2(lFx, lFy));
-                        spring_adjoint(e, k, lf.x, lf.y, lFz - gb.z, sc.x, sc.y, ldx, ldy, ldz, dk, da, db);
-                        lux -= ldx; luy -= ldy; luz -= ldz;
-                        sl[d * Ss + cidx] = make_float4(ldx, ldy, ldz, e.ext);
-                        __syncwarp();
-                        tmem_st4(tm + cells_s<d>(), cur[2], __float_as_uint(__uint_as_float(cur[3]) + dk),
-                                 __float_as_uint(__uint_as_float(cur[4]) + da),
-                                 __float_as_uint(__uint_as_float(cur[5]) + db));
-                    });
-                    tmem_wait_st();                       // the sums are read again next step
-                }
-                group_sync(bar, gthreads);
+                    tmem_st4(tm + cells_s<d>(), cur[2], __float_as_uint(__uint_as_float(cur[3]) + dk),
+                             __float_as_uint(__uint_as_float(cur[4]) + da),
+                             __float_as_uint(__uint_as_float(cur[5]) + db));
+                });
+                tmem_wait_st();                       // the sums are read again next step
+                flow.arrive_a();
+                if (!flow.wait_a(ph)) { atomicOr(a.status, 8); break; }
                 for_each_dir([&](auto t) {
                     constexpr int d = decltype(t)::value;
                     if (!((fl >> (16 + d)) & 1u)) return;
-                    const float4 ld = sl[d * Ss + cidx - lattice_offset<d>(Xs, XYs)];
+                    const int at = 13 * (row - lattice_offset<d>(RX, RXY)) + d;
+                    const float4 ld = GRID8 ? nl.load(at) : sl[at];
                     lux += ld.x; luy += ld.y; luz += ld.z;
                 });
             }
@@ -233,6 +248,9 @@ __global__ void __launch_bounds__(kBlock, 1) k_adjoint_lattice(AdjointArgs a)
             // scattered onto the voxels
             if (warp_in) {
                 const int64_t vo = a.pv.voff[r];
+                // opaque copies: the addresses formed here are not hoisted above the sweep and spilled
+                int ce = cidx, Ce = C;
+                asm volatile("" : "+r"(ce), "+r"(Ce));
                 for_each_dir([&](auto t) {
                     constexpr int d = decltype(t)::value;
                     uint32_t v6[6];
@@ -242,11 +260,11 @@ __global__ void __launch_bounds__(kBlock, 1) k_adjoint_lattice(AdjointArgs a)
                     if (!((fl >> d) & 1u)) return;
                     const float sk = __uint_as_float(v6[3]), sa = __uint_as_float(v6[4]), sbb = __uint_as_float(v6[5]);
                     if (!a.last) {
-                        accg[d * C + cidx] = sk;
-                        accg[(13 + d) * C + cidx] = sa;
-                        accg[(26 + d) * C + cidx] = sbb;
+                        accg[d * Ce + ce] = sk;
+                        accg[(13 + d) * Ce + ce] = sa;
+                        accg[(26 + d) * Ce + ce] = sbb;
                     } else {
-                        spring_sens_to_voxels<d>(cidx, X, XY, nx, ny, nz, a.mat + vo, sk, sa, sbb, c, a.g_k + vo,
+                        spring_sens_to_voxels<d>(ce, X, XY, nx, ny, nz, a.mat + vo, sk, sa, sbb, c, a.g_k + vo,
                                                  a.g_a + vo, a.g_b + vo);
                     }
                 });
@@ -290,7 +308,7 @@ __global__ void k_adjoint_voxels(const uint8_t* __restrict__ mat, const float* _
 
 cudaError_t launch_adjoint_lattice(const AdjointArgs& a, int grid, int threads, size_t smem, cudaStream_t s)
 {
-    auto kernel = a.cube8 ? k_adjoint_lattice<true> : k_adjoint_lattice<false>;
+    auto kernel = a.grid8 ? k_adjoint_lattice<true> : k_adjoint_lattice<false>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kernel<<<grid, threads, smem, s>>>(a);

@@ -150,7 +150,9 @@ struct voxsim_ctx {
     // (lattice items: the per-corner variant's first, n_items_corner of them, then the
     // direction-compacted variant's)
     int n_items = 0, n_items_corner = 0, n_big = 0, max_big_corner = 0;
-    bool has_split = false;        // some lattice items are split (two threads per corner)
+    // every lattice item is a single robot stepped with several threads per mass (step_roles.cu)
+    bool roles = false;
+    int roles_max_corner = 0;
     // mass-packed plan of the per-corner lattice robots (SIM_LATTICE_PACKED; used for stepping
     // that records nothing per step; the adjoint's replays run the per-corner plan, same bits)
     int n_pitems = 0;
@@ -191,7 +193,7 @@ struct voxsim_ctx {
     DevBuf<int> d_cluster;
     int n_stream = 0, max_stream_corner = 0;
     bool stream_cube40 = false;  // every streamed robot is 40 x 40 x 40
-    bool corner_cube8 = false;   // every per-corner lattice item is one 8 x 8 x 8 robot (768 threads)
+    bool corner_grid8 = false;   // every per-corner lattice item is one robot of at most 8 voxels per axis (768 threads)
     std::vector<int> stream_robots;
     DevBuf<int> d_stream;
     // CUDA graph of the streamed N-step loop, cached by step count (captured on a private
@@ -357,13 +359,14 @@ sim_status copy_out(void* dst, const void* src, size_t bytes, int mem, cudaStrea
 //   word 0 bit 0: the component labelling of a robot hit its iteration bound;
 //   word 0 bit 1: a material id of device-memory genomes was out of range (decoded as empty);
 //   word 1 bit 2: a bounded wait of the tensor-core MLP query gave up (the CTA aborted);
-//   word 2 bit 3: a segment of the per-corner lattice step gave up waiting for its robots'
-//   previous segment (read by sim_fitness into host memory).
+//   word 2 bit 3: a warp of a lattice step or of the adjoint's sweep gave up waiting for a
+//   neighbouring warp's data, or a segment for its robots' previous segment (read by sim_fitness
+//   into host memory).
 sim_status status_from_words(const int32_t* w)
 {
     if (w[2] & 8)
-        return fail(SIM_ETIMEOUT, "lattice step: a segment's bounded wait on its robots' previous segment "
-                                  "gave up (their state is invalid)");
+        return fail(SIM_ETIMEOUT, "lattice step: a bounded wait on a neighbouring warp's data or on the "
+                                  "robots' previous segment gave up (their state is invalid)");
     if (w[1] & 4)
         return fail(SIM_ETIMEOUT, "MLP query: a bounded wait on the tensor-core pipeline gave up "
                                   "(copies and MMAs drained, decoded materials invalid)");
@@ -688,7 +691,7 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
     const int block = lattice_max_threads();
     ++ctx->items_version;
     if (!ctx->tuned) default_choices(ctx);
-    ctx->has_split = false;
+    ctx->roles = false;
     ctx->max_big_corner = 0;
     ctx->max_big_spring_cap = 0;
     ctx->atomic_groups.clear();
@@ -798,28 +801,39 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
             auto& v = variant == 0 ? lattice[k] : lattice_sp[k];
             std::sort(v.begin(), v.end());
             const int per = std::min(block / kSlot[k], spread);
-            // a robot alone in its block gets a second thread per corner (split item) when the
-            // slot allows and the springs have dashpots: its step's chain of spring evaluations
-            // is cut from 13 to 7 (measured -14 % on the paper's 30 robots 5x5x5; without
-            // dashpots the split measured from -13 % to +27 %, so it is not used there)
-            const bool split = variant == 0 && per == 1 && 2 * kSlot[k] <= block && damped;
             for (size_t i = 0; i < v.size(); i += per) {
                 const int n = (int)std::min<size_t>(per, v.size() - i);
-                items.push_back(make_int4((int)robots.size(), n, split ? 2 * kSlot[k] : kSlot[k],
-                                          split ? 2 : variant));
+                items.push_back(make_int4((int)robots.size(), n, kSlot[k], variant));
                 for (int j = 0; j < n; ++j) robots.push_back(v[i + j].second);
             }
-            if (split && !v.empty()) ctx->has_split = true;
         }
     }
-    // the per-corner kernel's compile-time 8 x 8 x 8 instantiation applies when every one of its
-    // items is a single robot of that grid in a 768-thread slot
-    ctx->corner_cube8 = ctx->n_items_corner > 0;
-    for (int i = 0; i < ctx->n_items_corner && ctx->corner_cube8; ++i) {
+    // the per-corner kernel's compile-time strides apply when every one of its items is a single
+    // robot of at most 8 voxels along each axis in a 768-thread slot
+    ctx->corner_grid8 = ctx->n_items_corner > 0;
+    for (int i = 0; i < ctx->n_items_corner && ctx->corner_grid8; ++i) {
         const int4 it = items[i];
         const int r = robots[it.x];
-        ctx->corner_cube8 = it.y == 1 && it.z == 768 && it.w == 0 && ctx->dims[3 * r] == 8 &&
-                            ctx->dims[3 * r + 1] == 8 && ctx->dims[3 * r + 2] == 8;
+        ctx->corner_grid8 = it.y == 1 && it.z == 768 && it.w == 0 && ctx->dims[3 * r] <= 8 &&
+                            ctx->dims[3 * r + 1] <= 8 && ctx->dims[3 * r + 2] <= 8;
+    }
+    // several threads per mass (step_roles.cu) when every robot has a block to itself and the blocks
+    // fit the SMs at once: then a step's latency counts, not its throughput (250 robots 5x5x5, 500
+    // steps: 1.64 ms with one thread per mass, which shares an SM's issue slots better over two
+    // rounds of robots).  With dashpots two rounds still gain (250 robots 5x5x5: 2.22 -> 1.47 ms;
+    // 300 robots 7x7x7: 3.54 -> 2.65 ms), since the dashpot coefficients leave the steps too.
+    const int n_roles = ctx->n_items_corner;
+    if (n_roles > 0 && n_roles <= ctx->num_sms * (damped ? 2 : 1) && !ctx->imp_active &&
+        ctx->p.lattice != SIM_LATTICE_PACKED && (int)ctx->mass_count.size() == ctx->P) {
+        bool fit = true;
+        int corners = 0;
+        for (int i = 0; i < n_roles && fit; ++i) {
+            const int r = robots[items[i].x];
+            fit = items[i].y == 1 && ctx->mass_count[r] <= roles_max_masses();
+            corners = std::max(corners, (ctx->dims[3 * r] + 1) * (ctx->dims[3 * r + 1] + 1) * (ctx->dims[3 * r + 2] + 1));
+        }
+        ctx->roles = fit;
+        ctx->roles_max_corner = corners;
     }
     if (sim_status st = build_packed_items(ctx, lattice, mass_groups, damped)) return st;
     std::sort(atomic.begin(), atomic.end());
@@ -923,7 +937,7 @@ static sim_status build_packed_items(voxsim_ctx* ctx, const std::vector<std::vec
             }
         thin = n > (size_t)ctx->num_sms && slots > 0 && (double)used < 0.55 * (double)slots;
     }
-    const bool corner_too = masses_known && (ctx->p.lattice == SIM_LATTICE_PACKED || thin) && !ctx->has_split &&
+    const bool corner_too = masses_known && (ctx->p.lattice == SIM_LATTICE_PACKED || thin) && !ctx->roles &&
                             !ctx->imp_active;
     struct Grp { int T, C, r; };
     std::vector<Grp> gs;
@@ -1036,8 +1050,8 @@ static sim_status step_lattice(voxsim_ctx* ctx, int n, bool record)
     a.item_robots = ctx->d_item_robots.p;
     a.n_items = ctx->n_items;
     a.queue = ctx->d_queue.p;
-    a.has_split = ctx->has_split ? 1 : 0;
-    a.cube8 = ctx->corner_cube8 ? 1 : 0;
+    a.status = ctx->d_status.p + 2;
+    a.grid8 = ctx->corner_grid8 ? 1 : 0;
     ctx->imposed_args(a, ctx->step);
     if (record) {                               // (buffers sized by sim_step_n)
         a.ckpt_u = ctx->d_ckpt_u.p;
@@ -1051,7 +1065,6 @@ static sim_status step_lattice(voxsim_ctx* ctx, int n, bool record)
         }
     }
     const int threads = lattice_max_threads();
-    const size_t smem = sizeof(float4) * kLatticeSlotVec4 * (size_t)threads;
     VX_CK(cudaMemsetAsync(ctx->d_queue.p, 0, 2 * sizeof(int), ctx->stream));
     // per-corner variant: items [0, n_items_corner); direction-compacted variant: the rest
     const int n_corner = ctx->n_items_corner, n_spring = ctx->n_items - ctx->n_items_corner;
@@ -1071,7 +1084,6 @@ static sim_status step_lattice(voxsim_ctx* ctx, int n, bool record)
             b.nseg = nseg;
             b.seg_steps = (n + nseg - 1) / nseg;
             b.progress = ctx->d_progress.p;
-            b.status = ctx->d_status.p + 2;
             VX_CK(cudaMemsetAsync(b.progress, 0, sizeof(int) * ctx->n_pitems, ctx->stream));
         }
         VX_LAUNCH(ctx, launch_step_lattice_packed(b, std::min(ctx->n_pitems, ctx->num_sms), ctx->pitem_smem,
@@ -1080,17 +1092,17 @@ static sim_status step_lattice(voxsim_ctx* ctx, int n, bool record)
     if (n_corner > 0 && !(packed && ctx->pitems_cover_corner)) {
         a.n_items = n_corner;
         // (segmented instantiations exist for the undamped per-corner steps without imposed
-        // modes, recording only on 8 x 8 x 8 robots)
-        const bool seg_ok = !a.imp_modes && !a.c.damped && (!a.rec_u || ctx->corner_cube8);
-        const int nseg = seg_ok ? lattice_segments(n_corner, n, ctx->num_sms) : 1;
+        // modes, recording only on robots of at most 8 voxels along each axis)
+        const bool seg_ok = !a.imp_modes && !a.c.damped && (!a.rec_u || ctx->corner_grid8);
+        const int nseg = seg_ok && !ctx->roles ? lattice_segments(n_corner, n, ctx->num_sms) : 1;
         if (nseg > 1) {
             a.nseg = nseg;
             a.seg_steps = (n + nseg - 1) / nseg;
             a.progress = ctx->d_progress.p;
-            a.status = ctx->d_status.p + 2;
             VX_CK(cudaMemsetAsync(a.progress, 0, sizeof(int) * n_corner, ctx->stream));
         }
-        VX_LAUNCH(ctx, launch_step_lattice(a, std::min(n_corner, ctx->num_sms), threads, smem, ctx->stream));
+        if (ctx->roles) VX_LAUNCH(ctx, launch_step_roles(a, ctx->roles_max_corner, ctx->stream));
+        else VX_LAUNCH(ctx, launch_step_lattice(a, std::min(n_corner, ctx->num_sms), threads, ctx->stream));
         a.nseg = 0;
     }
     if (n_spring > 0) {
@@ -1099,7 +1111,7 @@ static sim_status step_lattice(voxsim_ctx* ctx, int n, bool record)
         a.queue = ctx->d_queue.p + 1;
         if (packed) VX_CK(cudaMemsetAsync(a.queue, 0, sizeof(int), ctx->stream));   // reused after the packed launch
         a.spack = ctx->d_spack.p;
-        VX_LAUNCH(ctx, launch_step_lattice(a, std::min(n_spring, ctx->num_sms), threads, smem, ctx->stream));
+        VX_LAUNCH(ctx, launch_step_lattice(a, std::min(n_spring, ctx->num_sms), threads, ctx->stream));
     }
     return SIM_OK;
 }
@@ -1117,7 +1129,7 @@ static sim_status step_cluster(voxsim_ctx* ctx, int n)
     a.sc = ctx->d_sc.p;
     a.nsteps = n;
     a.c = ctx->stepconst();
-    const size_t smem = sizeof(float4) * kLatticeSlotVec4 * (size_t)cluster_max_threads();
+    const size_t smem = sizeof(float4) * kSlotVec4 * (size_t)cluster_max_threads();
     for (const auto& g : ctx->cluster_groups) {
         a.robots = ctx->d_cluster.p + g.first;
         a.q = g.q;
@@ -1503,7 +1515,7 @@ static sim_status backward_lattice(voxsim_ctx* ctx, const double* dL_df)
         VX_CK(cudaStreamWaitEvent(r, ctx->ev_bwd[4], 0));
     }
     const int threads = lattice_max_threads();
-    const size_t smem = sizeof(float4) * kLatticeSlotVec4 * (size_t)threads;
+    const size_t smem = sizeof(float4) * kSlotVec4 * (size_t)threads;
     const int grid = std::min(ctx->n_items, ctx->num_sms);
     LatticeArgs f{};
     f.pv = ctx->view();
@@ -1514,8 +1526,9 @@ static sim_status backward_lattice(voxsim_ctx* ctx, const double* dL_df)
     f.items = ctx->d_items.p;
     f.item_robots = ctx->d_item_robots.p;
     f.n_items = ctx->n_items;
-    f.cube8 = ctx->corner_cube8 && ctx->n_items == ctx->n_items_corner ? 1 : 0;
+    f.grid8 = ctx->corner_grid8 && ctx->n_items == ctx->n_items_corner ? 1 : 0;
     f.queue = ctx->d_queue.p;
+    f.status = ctx->d_status.p + 2;
     f.rec_u = ctx->d_srec_u.p;
     f.rec_f = ctx->d_srec_f.p;
     f.rec_stride = (int64_t)Mc;
@@ -1538,8 +1551,9 @@ static sim_status backward_lattice(voxsim_ctx* ctx, const double* dL_df)
     a.items = ctx->d_items.p;
     a.item_robots = ctx->d_item_robots.p;
     a.n_items = ctx->n_items;
-    a.cube8 = f.cube8;
+    a.grid8 = f.grid8;
     a.queue = ctx->d_queue.p;
+    a.status = ctx->d_status.p + 2;
     a.g_k = ctx->d_gk.p;
     a.g_a = ctx->d_ga.p;
     a.g_b = ctx->d_gb.p;
@@ -1564,7 +1578,9 @@ static sim_status backward_lattice(voxsim_ctx* ctx, const double* dL_df)
             f.imp_step0 = ctx->rec_step0 + n0;
             f.queue = ctx->d_queue.p + 1;
             VX_CK(cudaMemsetAsync(f.queue, 0, sizeof(int), r));
-            VX_LAUNCH(ctx, launch_step_lattice(f, grid, threads, smem, r));
+            if (ctx->roles && ctx->n_items == ctx->n_items_corner)
+                VX_LAUNCH(ctx, launch_step_roles(f, ctx->roles_max_corner, r));
+            else VX_LAUNCH(ctx, launch_step_lattice(f, grid, threads, r));
             VX_CK(cudaEventRecord(ctx->ev_bwd[b], r));
             VX_CK(cudaStreamWaitEvent(s, ctx->ev_bwd[b], 0));
             a.rec_u = f.rec_u;
@@ -1708,8 +1724,9 @@ sim_status sim_get_contact_modes(voxsim_ctx* ctx, int32_t robot, uint8_t* out)
             f.items = ctx->d_items.p;
             f.item_robots = ctx->d_item_robots.p;
             f.n_items = ctx->n_items;
-            f.cube8 = ctx->corner_cube8 && ctx->n_items == ctx->n_items_corner ? 1 : 0;
+            f.grid8 = ctx->corner_grid8 && ctx->n_items == ctx->n_items_corner ? 1 : 0;
             f.queue = ctx->d_queue.p;
+            f.status = ctx->d_status.p + 2;
             f.rec_u = ctx->d_srec_u.p;
             f.rec_f = ctx->d_srec_f.p;
             f.rec_stride = (int64_t)Mc;
@@ -1724,8 +1741,7 @@ sim_status sim_get_contact_modes(voxsim_ctx* ctx, int32_t robot, uint8_t* out)
             ctx->imposed_args(f, ctx->rec_step0 + n0);
             const int threads = lattice_max_threads();
             VX_CK(cudaMemsetAsync(ctx->d_queue.p, 0, sizeof(int), s));
-            VX_LAUNCH(ctx, launch_step_lattice(f, std::min(ctx->n_items, ctx->num_sms), threads,
-                                               sizeof(float4) * kLatticeSlotVec4 * (size_t)threads, s));
+            VX_LAUNCH(ctx, launch_step_lattice(f, std::min(ctx->n_items, ctx->num_sms), threads, s));
         } else {
             StreamArgs f{};
             f.pv = ctx->view();

@@ -161,7 +161,7 @@ struct LatticeArgs {
     int nsteps;
     StepConst c;
     const int4* items;       // (first robot in item_robots, robots, threads per robot, kind:
-                             // 0 per corner, 1 direction-compacted, 2 per corner split); for the
+                             // 0 per corner, 1 direction-compacted); for the
                              // mass-packed kernel (first group in groups, groups, 0, 0)
     const int* item_robots;
     const int4* groups;      // mass-packed kernel: per group (robot, first thread, threads,
@@ -174,9 +174,9 @@ struct LatticeArgs {
     int nseg;
     int seg_steps;
     int* progress;
-    int* status;
-    int has_split;           // the items include split ones (run by the split instantiation)
-    int cube8;               // every per-corner item is one 8 x 8 x 8 robot in a 768-thread slot
+    int* status;             // (every lattice launch: the waits between warps report here too)
+    int grid8;               // every per-corner item is one robot of at most 8 voxels along each axis in a
+                             // 768-thread slot
     int* queue;              // work counter, zeroed before the launch
     // checkpoints for the adjoint (NULL when off): state at steps 0, K, 2K, ... of the call
     float4* ckpt_u;
@@ -298,8 +298,9 @@ struct AdjointArgs {
     const int4* items;
     const int* item_robots;
     int n_items;
-    int cube8;               // every item is one 8 x 8 x 8 robot in a 768-thread slot
+    int grid8;               // every item is one robot of at most 8 voxels along each axis in a 768-thread slot
     int* queue;
+    int* status;             // bit 3 set when a bounded wait between warps gave up
     float* g_k;              // per voxel: dL/dk_v, dL/d(alpha_v), dL/d(beta_v) accumulators
     float* g_a;
     float* g_b;
@@ -314,9 +315,12 @@ int lattice_max_threads();
 // Shared-memory bandwidth probe: grid blocks of 1024 threads, iters rounds of 8 16-byte loads.
 cudaError_t launch_probe_smem(int grid, int iters, float* sink, cudaStream_t s);
 size_t probe_smem_bytes_per_iter(int grid);
-constexpr int kLatticeSlotVec4 = 15;     // shared float4 per corner slot: u, v, 13 force planes
-cudaError_t launch_step_lattice(const LatticeArgs& a, int grid, int threads, size_t smem,
-                                cudaStream_t s);
+constexpr int kSlotVec4 = 15;            // shared float4 per corner slot: u, v, 13 force rows
+cudaError_t launch_step_lattice(const LatticeArgs& a, int grid, int threads, cudaStream_t s);
+// Several threads per mass, one block per item (each a single robot of at most roles_max_masses()
+// masses; max_corners: the largest robot's).
+int roles_max_masses();
+cudaError_t launch_step_roles(const LatticeArgs& a, int max_corners, cudaStream_t s);
 // Mass-packed lattice kernel: 768-thread blocks shared by groups of robots sized by mass count.
 cudaError_t launch_step_lattice_packed(const LatticeArgs& a, int grid, size_t smem, cudaStream_t s);
 size_t resident_smem_bytes(int max_mass, int max_spring_smem, int accumulate);

@@ -163,17 +163,36 @@ __device__ __forceinline__ void for_each_batch(F&& f)
     }
 }
 
+// Batches of up to B directions over D0 .. D1 - 1: f(first direction, count).
+template <int D0, int D1, int B, class F>
+__device__ __forceinline__ void for_each_batch_in(F&& f)
+{
+    if constexpr (D0 < D1) {
+        f(DirTag<D0>{}, DirTag<(D1 - D0 < B ? D1 - D0 : B)>{});
+        for_each_batch_in<D0 + B, D1, B>(f);
+    }
+}
+
 // Spring dashpot of the paper's preset (Table II spring damping ratio): adds
 // c_s ((v_b - v_a) . u) u to the force on a, c_s = spring_c sqrt(k) (spring_c = 2 zeta sqrt(m / 2)).
-__device__ __forceinline__ void spring_dashpot(SpringEval& e, float dvx, float dvy, float dvz, float k,
-                                               const StepConst& c)
+__device__ __forceinline__ float dashpot_coefficient(float k, const StepConst& c)
 {
-    const float cs = __fmul_rn(c.spring_c, __fsqrt_rn(k));
+    return __fmul_rn(c.spring_c, __fsqrt_rn(k));
+}
+
+__device__ __forceinline__ void spring_dashpot_c(SpringEval& e, float dvx, float dvy, float dvz, float cs)
+{
     const float rv = __fmul_rn(__fmaf_rn(e.dz, dvz, __fmaf_rn(e.dy, dvy, __fmul_rn(e.dx, dvx))), e.inv);
     const float fd = __fmul_rn(__fmul_rn(cs, rv), e.inv);      // per unit of d
     e.gx = __fmaf_rn(fd, e.dx, e.gx);
     e.gy = __fmaf_rn(fd, e.dy, e.gy);
     e.gz = __fmaf_rn(fd, e.dz, e.gz);
+}
+
+__device__ __forceinline__ void spring_dashpot(SpringEval& e, float dvx, float dvy, float dvz, float k,
+                                               const StepConst& c)
+{
+    spring_dashpot_c(e, dvx, dvy, dvz, dashpot_coefficient(k, c));
 }
 
 // Semi-implicit Euler with velocity damping, v <- c (v + dt F / m), u <- u + dt v, with the

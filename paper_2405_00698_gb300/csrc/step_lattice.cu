@@ -19,6 +19,8 @@
 // cancellation: l - L0 = (2 d0.du + du.du) / (l + L0).
 #include "common.cuh"
 #include "physics.cuh"
+#include "shared_rows.cuh"
+#include "warp_flow.cuh"
 
 namespace vx {
 namespace {
@@ -49,30 +51,30 @@ __device__ __forceinline__ void group_sync(int id, int nthreads)
 // keeps its registers).  RECORD: the adjoint's replay of a checkpoint segment, which also writes
 // every step's state before the update with its contact mode, and the horizontal spring force
 // before contact.
-// SPLIT (with dashpots): split items (item.w == 2: one robot of up to 384 corners alone in a
-// block, when the population leaves SMs idle) give every corner a second thread in another warp: the owner evaluates
-// directions 0..6, the helper directions 7..12 (writing their planes only), and after the
-// barrier the owner adds the helper's six plane entries in direction order before the backward
-// gather, so the sums are formed in the same order from the same values: the same bits as the
-// unsplit step, with the longest chain of spring evaluations per step cut from 13 to 7.
 // IMPOSE: some robots take their contact modes from a table (sim_impose_contact_modes).
-// CUBE8: every item of the launch is one 8 x 8 x 8 robot in a 768-thread slot (the MLP
-// population's fixed grid); the strides and the plane stride become compile-time constants, so
-// the shared-memory addresses of the 13 directions are immediate offsets.
-template <bool DAMPED, bool RECORD, bool SPLIT, bool IMPOSE, bool CUBE8 = false>
+// GRID8: every item of the launch is one robot of at most 8 voxels along each axis in a 768-thread
+// slot.  Its rows in shared memory lie as on the full 9 x 9 x 9 lattice of corners, so the strides
+// are compile-time constants and the addresses of the 13 directions immediate offsets; the rows
+// are the narrow ones, and the warps wait for their neighbours (WarpFlow) instead of for the
+// group: 1024 MLP robots 8x8x8, 2000 steps: 32.8 ms with the group's barriers and float4 rows in
+// 13 planes, 31.7 ms with narrow rows, 29.9 ms with the neighbour waits too.  With run-time strides
+// the neighbour waits measured within 1 % of the barriers (12 % slower on groups of four warps),
+// narrow rows slower.
+template <bool DAMPED, bool RECORD, bool IMPOSE, bool GRID8 = false>
 __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice(LatticeArgs a)
 {
-    extern __shared__ __align__(16) float4 sm4[];
-    __shared__ int sh_item[5];
+    __shared__ int sh_item[4];
+    __shared__ FlowBars sh_flow;
+    float4* const sm4 = reinterpret_cast<float4*>(lattice_smem);
     const int tid = threadIdx.x;
     const StepConst c = a.c;
+    flow_create(sh_flow);
     for (;;) {
         if (tid == 0) {
             const int it = atomicAdd(a.queue, 1);
             if (it < a.n_items) {
                 const int4 item = a.items[it];
                 sh_item[0] = item.x; sh_item[1] = item.y; sh_item[2] = item.z; sh_item[3] = 1;
-                sh_item[4] = item.w;
             } else {
                 sh_item[3] = 0;
             }
@@ -80,56 +82,63 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice(LatticeA
         __syncthreads();
         if (!sh_item[3]) break;
         const int first = sh_item[0], count = sh_item[1], gthreads = sh_item[2];
-        // split groups only in the SPLIT instantiation (launched when the plan has some); the
-        // other instantiations run a split item as one unsplit group of 2 S threads
-        const bool split = SPLIT && sh_item[4] == 2;
-        const int group = CUBE8 ? 0 : tid / gthreads, lt = CUBE8 ? tid : tid % gthreads;
+        const int group = GRID8 ? 0 : tid / gthreads, lt = GRID8 ? tid : tid % gthreads;
         __syncthreads();   // everyone has read the item before thread 0 may overwrite it
         if (group < count) {
             const int r = a.item_robots[first + group];
             const int nx = a.pv.dims[3 * r], ny = a.pv.dims[3 * r + 1], nz = a.pv.dims[3 * r + 2];
-            const int X = CUBE8 ? 9 : nx + 1, XY = CUBE8 ? 81 : (nx + 1) * (ny + 1), C = CUBE8 ? 729 : XY * (nz + 1);
+            const int X = nx + 1, XY = X * (ny + 1), C = XY * (nz + 1);
+            // row strides in shared memory: the grid's own, or those of 9 x 9 x 9 corners
+            const int RX = GRID8 ? 9 : X, RXY = GRID8 ? 81 : XY;
             const int64_t mo = a.pv.moff[r];
             const int bar = 1 + group;
-            // shared-memory slot of this group (S corners): u, then 13 force planes; a split
-            // group has 2 S threads, owners [0, S) and helpers [S, 2 S) (whole warps each)
-            const int S = CUBE8 ? kMaxLatticeThreads : (split ? gthreads / 2 : gthreads);
-            const bool hlp = split && lt >= S;
-            const int li = hlp ? lt - S : lt;
-            float4* su = sm4 + (size_t)group * kLatticeSlotVec4 * S;
+            // shared-memory slot of this group (S corners): u, v, then 13 force rows per corner
+            // (row 13 a + d: force on a of spring (a, d))
+            const int S = GRID8 ? kMaxLatticeThreads : gthreads;
+            float4* su = sm4 + (size_t)group * kSlotVec4 * S;
             float4* sv = su + S;               // velocities (read by spring dashpots)
-            float4* fb = sv + S;               // plane d at fb + d * S: force on a of spring (a, d)
-            // thread li owns the li-th mass (ascending corner order: neighbouring threads touch
+            float4* fb = sv + S;
+            const NarrowRows nu(0, kMaxLatticeThreads), nf(12 * kMaxLatticeThreads, 13 * kMaxLatticeThreads);   // GRID8
+            // thread lt owns the lt-th mass (ascending corner order: neighbouring threads touch
             // neighbouring shared-memory rows); threads past the mass count only take part in the
             // barriers
             const int M = a.pv.n_mass[r];
-            const bool in = li < M;
-            const int cidx = in ? a.corner_order[mo + li] : 0;
+            const bool in = lt < M;
+            const int cidx = in ? a.corner_order[mo + lt] : 0;
+            const int row = GRID8 ? cidx + (cidx / X) * (9 - X) + (cidx / XY) * (81 - 9 * (ny + 1)) : cidx;
             const uint32_t fl = in ? a.cflags[mo + cidx] : 0u;
             float pk[13], pa[13], pb[13];
             const float* prm = a.prm + 39 * mo;
             for_each_dir([&](auto t) {
                 constexpr int d = decltype(t)::value;
-                const bool has = ((fl >> d) & 1u) && (!split || hlp == (d >= 7));
+                const bool has = (fl >> d) & 1u;
                 pk[d] = has ? prm[(0 * 13 + d) * C + cidx] : 0.f;
                 pa[d] = has ? prm[(1 * 13 + d) * C + cidx] : 0.f;
                 pb[d] = has ? prm[(2 * 13 + d) * C + cidx] : 0.f;
             });
             float4 u = in ? a.u[mo + cidx] : make_float4(0.f, 0.f, 0.f, 0.f);
             float4 v = in ? a.v[mo + cidx] : make_float4(0.f, 0.f, 0.f, 0.f);
-            const bool mass = ((fl >> 31) & 1u) && !hlp;
+            const bool mass = (fl >> 31) & 1u;
             const int64_t imp = IMPOSE ? a.imp_off[r] : -1;
-            if (in && !hlp) {
-                su[cidx] = u;
+            auto put_u = [&] {
+                if constexpr (GRID8) nu.store(row, u.x, u.y, u.z);
+                else su[cidx] = u;
+            };
+            if (in) {
+                put_u();
                 if (DAMPED) sv[cidx] = v;
             }
+            // whole warps past the masses take no part in the steps
+            const bool warp_in = (lt & ~31) < M;
+            const int nw = (M + 31) >> 5;
+            WarpFlow flow;
+            if (GRID8 && warp_in) flow.init(sh_flow, 0, lt >> 5, nw, 91);
             group_sync(bar, gthreads);
-            for (int n = 0; n < a.nsteps; ++n) {
-                if (hlp && in) {                   // the owner's state after the previous step
-                    u = su[cidx];
-                    if (DAMPED) v = sv[cidx];
-                }
-                if (a.ckpt_u && in && !hlp && n % a.ckpt_every == 0) {   // state at the start of segment n / K
+            // a warp of the top layer has no springs upwards: it skips those directions (1 %)
+            const bool up = __any_sync(0xffffffffu, fl & 0x1ff0u);
+            uint32_t ph = 0;
+            if (warp_in) for (int n = 0; n < a.nsteps; ++n, ph ^= 1u) {
+                if (a.ckpt_u && in && n % a.ckpt_every == 0) {   // state at the start of segment n / K
                     const int64_t o = (int64_t)(n / a.ckpt_every) * a.ckpt_stride + mo + cidx;
                     a.ckpt_u[o] = u;
                     a.ckpt_v[o] = v;
@@ -142,9 +151,8 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice(LatticeA
                 // (du = 0, so ext = 0 and the force is an exact zero that leaves the sums' bits
                 // unchanged); its plane entry is never read.  6.5 % faster than skipping it, and
                 // 2.6 % more with the far end's load predicated off (u from the register).
-                if (in) for_each_dir([&](auto t) {
+                auto forward = [&](auto t) {
                     constexpr int d = decltype(t)::value;
-                    if (split && hlp != (d >= 7)) return;   // the other thread's direction
                     const bool has = (fl >> d) & 1u;
                     if constexpr (DAMPED) {
                         // with dashpots an absent spring would also load a velocity and take a
@@ -152,31 +160,33 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice(LatticeA
                         if (!has) return;
                     }
                     float4 ub = u;
-                    if (has) ub = su[cidx + lattice_offset<d>(X, XY)];
+                    if (has) ub = GRID8 ? nu.load(row + lattice_offset<d>(RX, RXY)) : su[row + lattice_offset<d>(RX, RXY)];
                     SpringEval e = spring_eval_ends<d>(ub, u, c.edge, lattice_rest<d>(c), lattice_rest_sq<d>(c),
                                                       pk[d], pa[d], pb[d], sc.x, sc.y);
                     if constexpr (DAMPED) {
-                        const float4 vb = sv[has ? cidx + lattice_offset<d>(X, XY) : cidx];
+                        const float4 vb = sv[has ? row + lattice_offset<d>(RX, RXY) : cidx];
                         spring_dashpot(e, __fsub_rn(vb.x, v.x), __fsub_rn(vb.y, v.y), __fsub_rn(vb.z, v.z), pk[d], c);
                     }
                     Fxy = __fadd2_rn(Fxy, make_float2(e.gx, e.gy)); Fz = __fadd_rn(Fz, e.gz);
-                    // the plane's fourth lane is never read: it takes a value already in a
-                    // register (the extension) rather than a zero (2.3 % fewer instructions)
-                    fb[d * S + cidx] = make_float4(e.gx, e.gy, e.gz, e.ext);
-                });
-                group_sync(bar, gthreads);
-                // phase B (owners): the helper's forward springs in direction order, then the
-                // backward springs (c - offset(d), c), then the mass update
-                if (split && in && !hlp) for_each_dir_in<7, 6>([&](auto t) {
-                    constexpr int d = decltype(t)::value;
-                    if (!((fl >> d) & 1u)) return;
-                    const float4 g = fb[d * S + cidx];
-                    Fxy = __fadd2_rn(Fxy, make_float2(g.x, g.y)); Fz = __fadd_rn(Fz, g.z);
-                });
-                if (!hlp) for_each_dir([&](auto t) {
+                    if constexpr (GRID8) nf.store(13 * row + d, e.gx, e.gy, e.gz);
+                    else fb[13 * row + d] = make_float4(e.gx, e.gy, e.gz, e.ext);   // (any value in the unused lane)
+                };
+                if (in) {
+                    for_each_dir_in<0, 4>(forward);
+                    if (!GRID8 || up) for_each_dir_in<4, 9>(forward);
+                }
+                if constexpr (GRID8) {
+                    flow.arrive_a();
+                    if (!flow.wait_a(ph)) { atomicOr(a.status, 8); break; }
+                } else {
+                    group_sync(bar, 32 * nw);
+                }
+                // phase B: the backward springs (c - offset(d), c), then the mass update
+                for_each_dir([&](auto t) {
                     constexpr int d = decltype(t)::value;
                     if (!((fl >> (16 + d)) & 1u)) return;
-                    const float4 g = fb[d * S + cidx - lattice_offset<d>(X, XY)];   // force on a
+                    const int at = 13 * (row - lattice_offset<d>(RX, RXY)) + d;
+                    const float4 g = GRID8 ? nf.load(at) : fb[at];   // force on a
                     Fxy = __ffma2_rn(make_float2(g.x, g.y), kMinusOne2, Fxy); Fz = __fsub_rn(Fz, g.z);
                 });
                 if (mass) {
@@ -197,12 +207,17 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice(LatticeA
                     } else {
                         mass_update(u, v, Fxy.x, Fxy.y, Fz, c);
                     }
-                    su[cidx] = u;
+                    put_u();
                     if (DAMPED) sv[cidx] = v;
                 }
-                group_sync(bar, gthreads);
+                if constexpr (GRID8) {
+                    flow.arrive_b();
+                    if (!flow.wait_b(ph)) { atomicOr(a.status, 8); break; }
+                } else {
+                    group_sync(bar, 32 * nw);
+                }
             }
-            if (in && !hlp) {
+            if (in) {
                 a.u[mo + cidx] = u;
                 a.v[mo + cidx] = v;
             }
@@ -213,8 +228,8 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice(LatticeA
 
 
 // ----------------------------------------------------------------------------------------------
-// Segmented queue for the per-corner step (undamped, no split items, no imposed modes; RECORD as
-// above; CUBE8 as above).  With more items than SMs a queue of whole items leaves SMs idle while
+// Segmented queue for the per-corner step (undamped, no imposed modes; RECORD as
+// above; GRID8 as above).  With more items than SMs a queue of whole items leaves SMs idle while
 // the last wave's robots run all their steps; here every item's steps are cut into a.nseg
 // segments of a.seg_steps and the queue holds the (segment, item) units in segment-major order,
 // so the last wave waits for one segment.  A unit first waits (thread 0, bounded) until its item's
@@ -226,14 +241,16 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice(LatticeA
 // one unit per item (tested).  A separate kernel rather than a template switch of the one above:
 // with the switch, the unsegmented instantiations measured 2 % slower.
 // ----------------------------------------------------------------------------------------------
-template <bool RECORD, bool CUBE8>
+template <bool RECORD, bool GRID8>
 __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_seg(LatticeArgs a)
 {
-    extern __shared__ __align__(16) float4 sm4[];
     // item (first robot, robots, threads), more work, -, segment, item index, segment's end
     __shared__ int sh_item[8];
+    __shared__ FlowBars sh_flow;
+    float4* const sm4 = reinterpret_cast<float4*>(lattice_smem);
     const int tid = threadIdx.x;
     const StepConst c = a.c;
+    flow_create(sh_flow);
     for (;;) {
         if (tid == 0) {
             const int it = atomicAdd(a.queue, 1);
@@ -258,20 +275,24 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_seg(Latt
         if (!sh_item[3]) break;
         const int first = sh_item[0], count = sh_item[1], gthreads = sh_item[2];
         const int n_begin = sh_item[5] * a.seg_steps;
-        const int group = CUBE8 ? 0 : tid / gthreads, lt = CUBE8 ? tid : tid % gthreads;
+        const int group = GRID8 ? 0 : tid / gthreads, lt = GRID8 ? tid : tid % gthreads;
         __syncthreads();   // everyone has read the item before thread 0 may overwrite it
         if (group < count) {
             const int r = a.item_robots[first + group];
             const int nx = a.pv.dims[3 * r], ny = a.pv.dims[3 * r + 1], nz = a.pv.dims[3 * r + 2];
-            const int X = CUBE8 ? 9 : nx + 1, XY = CUBE8 ? 81 : (nx + 1) * (ny + 1), C = CUBE8 ? 729 : XY * (nz + 1);
+            const int X = nx + 1, XY = X * (ny + 1), C = XY * (nz + 1);
+            // row strides in shared memory: the grid's own, or those of 9 x 9 x 9 corners
+            const int RX = GRID8 ? 9 : X, RXY = GRID8 ? 81 : XY;
             const int64_t mo = a.pv.moff[r];
             const int bar = 1 + group;
-            const int S = CUBE8 ? kMaxLatticeThreads : gthreads;   // (a split item: one group of 2 S)
-            float4* su = sm4 + (size_t)group * kLatticeSlotVec4 * S;
-            float4* fb = su + 2 * S;           // plane d at fb + d * S (after u and the unused v)
+            const int S = GRID8 ? kMaxLatticeThreads : gthreads;
+            float4* su = sm4 + (size_t)group * kSlotVec4 * S;
+            float4* fb = su + 2 * S;           // (after u and the unused v)
+            const NarrowRows nu(0, kMaxLatticeThreads), nf(12 * kMaxLatticeThreads, 13 * kMaxLatticeThreads);   // GRID8
             const int M = a.pv.n_mass[r];
             const bool in = lt < M;
             const int cidx = in ? a.corner_order[mo + lt] : 0;
+            const int row = GRID8 ? cidx + (cidx / X) * (9 - X) + (cidx / XY) * (81 - 9 * (ny + 1)) : cidx;
             const uint32_t fl = in ? a.cflags[mo + cidx] : 0u;
             float pk[13], pa[13], pb[13];
             const float* prm = a.prm + 39 * mo;
@@ -286,11 +307,22 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_seg(Latt
             float4 u = in ? __ldcg(a.u + mo + cidx) : make_float4(0.f, 0.f, 0.f, 0.f);
             float4 v = in ? __ldcg(a.v + mo + cidx) : make_float4(0.f, 0.f, 0.f, 0.f);
             const bool mass = (fl >> 31) & 1u;
-            if (in) su[cidx] = u;
+            auto put_u = [&] {
+                if constexpr (GRID8) nu.store(row, u.x, u.y, u.z);
+                else su[cidx] = u;
+            };
+            if (in) put_u();
+            const bool warp_in = (lt & ~31) < M;
+            const int nw = (M + 31) >> 5;
+            WarpFlow flow;
+            if (GRID8 && warp_in) flow.init(sh_flow, 0, lt >> 5, nw, 91);
             group_sync(bar, gthreads);
+            // a warp of the top layer has no springs upwards: it skips those directions (1 %)
+            const bool up = __any_sync(0xffffffffu, fl & 0x1ff0u);
+            uint32_t ph = 0;
             // (the segment's end is re-read from shared memory each step rather than held in a
             // register through the step)
-            for (int n = n_begin; n < *(volatile int*)&sh_item[7]; ++n) {
+            if (warp_in) for (int n = n_begin; n < *(volatile int*)&sh_item[7]; ++n, ph ^= 1u) {
                 if (a.ckpt_u && in && n % a.ckpt_every == 0) {   // state at the start of segment n / K
                     const int64_t o = (int64_t)(n / a.ckpt_every) * a.ckpt_stride + mo + cidx;
                     a.ckpt_u[o] = u;
@@ -300,22 +332,33 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_seg(Latt
                 float2 Fxy = make_float2(0.f, 0.f);
                 float Fz = 0.f;
                 // phase A: forward springs, branch-free (an absent spring is an exact zero force)
-                if (in) for_each_dir([&](auto t) {
+                auto forward = [&](auto t) {
                     constexpr int d = decltype(t)::value;
                     const bool has = (fl >> d) & 1u;
                     float4 ub = u;
-                    if (has) ub = su[cidx + lattice_offset<d>(X, XY)];
+                    if (has) ub = GRID8 ? nu.load(row + lattice_offset<d>(RX, RXY)) : su[row + lattice_offset<d>(RX, RXY)];
                     SpringEval e = spring_eval_ends<d>(ub, u, c.edge, lattice_rest<d>(c), lattice_rest_sq<d>(c),
                                                       pk[d], pa[d], pb[d], sc.x, sc.y);
                     Fxy = __fadd2_rn(Fxy, make_float2(e.gx, e.gy)); Fz = __fadd_rn(Fz, e.gz);
-                    fb[d * S + cidx] = make_float4(e.gx, e.gy, e.gz, e.ext);
-                });
-                group_sync(bar, gthreads);
+                    if constexpr (GRID8) nf.store(13 * row + d, e.gx, e.gy, e.gz);
+                    else fb[13 * row + d] = make_float4(e.gx, e.gy, e.gz, e.ext);   // (any value in the unused lane)
+                };
+                if (in) {
+                    for_each_dir_in<0, 4>(forward);
+                    if (!GRID8 || up) for_each_dir_in<4, 9>(forward);
+                }
+                if constexpr (GRID8) {
+                    flow.arrive_a();
+                    if (!flow.wait_a(ph)) { atomicOr(a.status, 8); break; }
+                } else {
+                    group_sync(bar, 32 * nw);
+                }
                 // phase B: backward springs in direction order, then the mass update
                 if (in) for_each_dir([&](auto t) {
                     constexpr int d = decltype(t)::value;
                     if (!((fl >> (16 + d)) & 1u)) return;
-                    const float4 g = fb[d * S + cidx - lattice_offset<d>(X, XY)];   // force on a
+                    const int at = 13 * (row - lattice_offset<d>(RX, RXY)) + d;
+                    const float4 g = GRID8 ? nf.load(at) : fb[at];   // force on a
                     Fxy = __ffma2_rn(make_float2(g.x, g.y), kMinusOne2, Fxy); Fz = __fsub_rn(Fz, g.z);
                 });
                 if (mass) {
@@ -328,9 +371,14 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_seg(Latt
                     } else {
                         mass_update(u, v, Fxy.x, Fxy.y, Fz, c);
                     }
-                    su[cidx] = u;
+                    put_u();
                 }
-                group_sync(bar, gthreads);
+                if constexpr (GRID8) {
+                    flow.arrive_b();
+                    if (!flow.wait_b(ph)) { atomicOr(a.status, 8); break; }
+                } else {
+                    group_sync(bar, 32 * nw);
+                }
             }
             if (in) {
                 a.u[mo + cidx] = u;
@@ -390,7 +438,7 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_compact(
             const int64_t mo = a.pv.moff[r];
             const int bar = 1 + group;
             const int S = gthreads;
-            float4* su = sm4 + (size_t)group * kLatticeSlotVec4 * S;
+            float4* su = sm4 + (size_t)group * kSlotVec4 * S;
             float4* sv = su + S;
             float4* fb = sv + S;
             int* nd = sh_nd[group];
@@ -501,7 +549,7 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_compact(
 // memory is indexing the force planes by the thread slot of the spring's far end (the reader)
 // instead of by corner: a robot needs 13 planes of T entries (T = its threads) and its
 // displacements by corner (C entries), not 13 planes of C entries.  The far end's slot rides in
-// the .w lane of its shared displacement, which the spring evaluation loads anyway.
+// an integer beside the z of its shared displacement, which the spring evaluation loads anyway.
 // Per step:
 //   phase A: for each forward spring (c, c + off(d)) the owner computes the force f from its own
 //            displacement and the far end's, adds f to its own total, and writes f into plane d
@@ -511,14 +559,12 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_compact(
 // The sums run over the same values in the same order as the per-corner kernel (own forward
 // springs by direction, then backward springs by direction): identical bits, so the adjoint's
 // replay (which runs the per-corner kernel) reproduces a run of this one.
-// Shared memory of a group: C float4 displacements (+ C velocities with dashpots), 13 T float4
-// plane entries, 32 float4 rows for absent springs.
 // ----------------------------------------------------------------------------------------------
 template <bool DAMPED>
 __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_packed(LatticeArgs a)
 {
-    extern __shared__ __align__(16) float4 sm4[];
     __shared__ int sh_item[3];
+    float4* const sm4 = reinterpret_cast<float4*>(lattice_smem);
     const int tid = threadIdx.x;
     const StepConst c = a.c;
     for (;;) {
@@ -549,16 +595,16 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_packed(L
             const int X = nx + 1, XY = (nx + 1) * (ny + 1), C = XY * (nz + 1);
             const int64_t mo = a.pv.moff[r];
             const int bar = 1 + group;
-            float4* su = sm4 + gi.w;                 // displacements by corner, slot id in .w
-            float4* sv = su + C;                     // velocities by corner (dashpots only)
-            float4* fb = DAMPED ? sv + C : su + C;   // plane d at fb + d * T, by the reader's slot;
-                                                     // then 32 rows for absent springs (never read)
+            float4* su = sm4 + gi.w;                 // displacements by corner, slot in .w
+            float4* fb = su + C;                     // row 13 t + d: thread t's backward spring d; then 32
+                                                     // rows for absent springs (never read)
+            float4* sv = fb + 13 * T + 32;           // velocities by corner (dashpots only)
             const int M = a.pv.n_mass[r];
             const bool in = lt < M;
             const int cidx = in ? a.corner_order[mo + lt] : 0;
             const uint32_t fl = in ? a.cflags[mo + cidx] : 0u;
-            const float slot = __int_as_float(lt);
-            const int junk = 13 * T + (lt & 31);     // this lane's row for absent springs
+            const float slot = __int_as_float(13 * lt);   // this thread's first force row
+            const int junk = 13 * T + (lt & 31);          // this lane's row for absent springs
             float pk[13], pa[13], pb[13];
             const float* prm = a.prm + 39 * mo;
             for_each_dir([&](auto t) {
@@ -586,7 +632,7 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_packed(L
                 float Fz = 0.f;
                 // phase A: forward springs, no branch per direction (an absent spring has zero
                 // parameters and the corner itself as far end: an exact zero force)
-                if (in) for_each_dir([&](auto t) {
+                auto forward = [&](auto t) {
                     constexpr int d = decltype(t)::value;
                     const bool has = (fl >> d) & 1u;
                     if constexpr (DAMPED) {
@@ -601,16 +647,17 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_packed(L
                         spring_dashpot(e, __fsub_rn(vb.x, v.x), __fsub_rn(vb.y, v.y), __fsub_rn(vb.z, v.z), pk[d], c);
                     }
                     Fxy = __fadd2_rn(Fxy, make_float2(e.gx, e.gy)); Fz = __fadd_rn(Fz, e.gz);
-                    const int row = has ? d * T + __float_as_int(ub.w) : junk;
+                    const int row = has ? __float_as_int(ub.w) + d : junk;
                     fb[row] = make_float4(e.gx, e.gy, e.gz, e.ext);
-                });
+                };
+                if (in) for_each_dir(forward);
                 group_sync(bar, T);
                 // phase B: backward springs (c - offset(d), c) from this slot's rows, then the update
                 if (in) {
                     for_each_dir([&](auto t) {
                         constexpr int d = decltype(t)::value;
                         if (!((fl >> (16 + d)) & 1u)) return;
-                        const float4 g = fb[d * T + lt];   // force on the spring's first end
+                        const float4 g = fb[13 * lt + d];   // force on the spring's first end
                         Fxy = __ffma2_rn(make_float2(g.x, g.y), kMinusOne2, Fxy); Fz = __fsub_rn(Fz, g.z);
                     });
                     if ((fl >> 31) & 1u) {
@@ -638,9 +685,9 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_packed(L
 // ----------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_packed_seg(LatticeArgs a)
 {
-    extern __shared__ __align__(16) float4 sm4[];
     // item (first group, groups), more work, -, -, segment, item index, segment's end
     __shared__ int sh_item[8];
+    float4* const sm4 = reinterpret_cast<float4*>(lattice_smem);
     const int tid = threadIdx.x;
     const StepConst c = a.c;
     for (;;) {
@@ -680,15 +727,14 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_packed_s
             const int X = nx + 1, XY = (nx + 1) * (ny + 1), C = XY * (nz + 1);
             const int64_t mo = a.pv.moff[r];
             const int bar = 1 + group;
-            float4* su = sm4 + gi.w;                 // displacements by corner, slot id in .w
-            float4* fb = su + C;                     // plane d at fb + d * T, by the reader's slot;
-                                                     // then 32 rows for absent springs (never read)
+            float4* su = sm4 + gi.w;                 // (as in k_step_lattice_packed)
+            float4* fb = su + C;
             const int M = a.pv.n_mass[r];
             const bool in = lt < M;
             const int cidx = in ? a.corner_order[mo + lt] : 0;
             const uint32_t fl = in ? a.cflags[mo + cidx] : 0u;
-            const float slot = __int_as_float(lt);
-            const int junk = 13 * T + (lt & 31);     // this lane's row for absent springs
+            const float slot = __int_as_float(13 * lt);   // this thread's first force row
+            const int junk = 13 * T + (lt & 31);          // this lane's row for absent springs
             float pk[13], pa[13], pb[13];
             const float* prm = a.prm + 39 * mo;
             for_each_dir([&](auto t) {
@@ -712,7 +758,7 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_packed_s
                 const float2 sc = a.sc[n];
                 float2 Fxy = make_float2(0.f, 0.f);
                 float Fz = 0.f;
-                if (in) for_each_dir([&](auto t) {
+                auto forward = [&](auto t) {
                     constexpr int d = decltype(t)::value;
                     const bool has = (fl >> d) & 1u;
                     float4 ub = u;
@@ -720,15 +766,16 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_packed_s
                     SpringEval e = spring_eval_ends<d>(ub, u, c.edge, lattice_rest<d>(c), lattice_rest_sq<d>(c),
                                                       pk[d], pa[d], pb[d], sc.x, sc.y);
                     Fxy = __fadd2_rn(Fxy, make_float2(e.gx, e.gy)); Fz = __fadd_rn(Fz, e.gz);
-                    const int row = has ? d * T + __float_as_int(ub.w) : junk;
+                    const int row = has ? __float_as_int(ub.w) + d : junk;
                     fb[row] = make_float4(e.gx, e.gy, e.gz, e.ext);
-                });
+                };
+                if (in) for_each_dir(forward);
                 group_sync(bar, T);
                 if (in) {
                     for_each_dir([&](auto t) {
                         constexpr int d = decltype(t)::value;
                         if (!((fl >> (16 + d)) & 1u)) return;
-                        const float4 g = fb[d * T + lt];   // force on the spring's first end
+                        const float4 g = fb[13 * lt + d];   // force on the spring's first end
                         Fxy = __ffma2_rn(make_float2(g.x, g.y), kMinusOne2, Fxy); Fz = __fsub_rn(Fz, g.z);
                     });
                     if ((fl >> 31) & 1u) {
@@ -764,26 +811,25 @@ cudaError_t launch_step_lattice_packed(const LatticeArgs& a, int grid, size_t sm
     return cudaGetLastError();
 }
 
-cudaError_t launch_step_lattice(const LatticeArgs& a, int grid, int threads, size_t smem,
-                                cudaStream_t s)
+cudaError_t launch_step_lattice(const LatticeArgs& a, int grid, int threads, cudaStream_t s)
 {
-    const bool cube8 = a.cube8 && !a.c.damped;
+    size_t smem = sizeof(float4) * kSlotVec4 * (size_t)threads;
+    const bool grid8 = a.grid8 && !a.c.damped;
     // a segmented queue (a.nseg > 1; the host sets it only for undamped per-corner items without
-    // imposed modes, recording only on 8 x 8 x 8 robots)
+    // imposed modes, recording only on robots of at most 8 voxels along each axis)
     if (a.nseg > 1) {
         auto kseg = a.rec_u ? k_step_lattice_seg<true, true>
-                  : (cube8 ? k_step_lattice_seg<false, true> : k_step_lattice_seg<false, false>);
+                  : (grid8 ? k_step_lattice_seg<false, true> : k_step_lattice_seg<false, false>);
         cudaError_t e = cudaFuncSetAttribute(kseg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         kseg<<<grid, threads, smem, s>>>(a);
         return cudaGetLastError();
     }
-    auto kernel = a.imp_modes ? (a.rec_u ? k_step_lattice<false, true, false, true> : k_step_lattice<false, false, false, true>)
-                : a.rec_u ? (cube8 ? k_step_lattice<false, true, false, false, true> : k_step_lattice<false, true, false, false>)
-                : (cube8 && !a.spack) ? k_step_lattice<false, false, false, false, true>
+    auto kernel = a.imp_modes ? (a.rec_u ? k_step_lattice<false, true, true> : k_step_lattice<false, false, true>)
+                : a.rec_u ? (grid8 ? k_step_lattice<false, true, false, true> : k_step_lattice<false, true, false>)
+                : (grid8 && !a.spack) ? k_step_lattice<false, false, false, true>
                 : a.spack ? (a.c.damped ? k_step_lattice_compact<true> : k_step_lattice_compact<false>)
-                : a.c.damped ? (a.has_split ? k_step_lattice<true, false, true, false> : k_step_lattice<true, false, false, false>)
-                             : k_step_lattice<false, false, false, false>;
+                : a.c.damped ? k_step_lattice<true, false, false> : k_step_lattice<false, false, false>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kernel<<<grid, threads, smem, s>>>(a);
