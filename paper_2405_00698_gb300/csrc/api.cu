@@ -222,7 +222,7 @@ struct voxsim_ctx {
     // device buffers
     DevBuf<int> d_dims;
     DevBuf<int64_t> d_voff, d_moff, d_soff, d_tmp_off;
-    DevBuf<int> d_nm, d_ns, d_lpt, d_queue, d_status, d_item_robots, d_big, d_grad_rows;
+    DevBuf<int> d_nm, d_ns, d_queue, d_status, d_item_robots, d_big, d_grad_rows;
     DevBuf<int> d_progress;      // per lattice item: segments done (segmented queue)
     DevBuf<int4> d_items;
     DevBuf<uint32_t> d_cflags;
@@ -233,11 +233,19 @@ struct voxsim_ctx {
     // sim_set_population copied from host memory into d_in_f32 (0: none), which evo_generation
     // can take as its input instead of a second upload
     int64_t host_genome_floats = 0;
-    DevBuf<int> d_label, d_count, d_corner_mass, d_mass_corner;
+    DevBuf<int> d_label, d_count, d_corner_mass, d_corner_spring, d_mass_corner;
+    // topology scratch: voxel parameters, large robots' list, totals and chunk counts
+    DevBuf<float4> d_vox_q;
+    DevBuf<float> d_vox_s;
+    DevBuf<int> d_topo_robots, d_zmin;
+    DevBuf<unsigned long long> d_best;
+    DevBuf<int2> d_chunk;
+    std::vector<int> topo_robots;   // (host copy of d_topo_robots: small robots, then large ones)
     DevBuf<int2> d_sab;
     DevBuf<float4> d_sp, d_spack, d_x0, d_x, d_v, d_x_alt, d_v_alt;
     DevBuf<float> d_plain_f;       // force accumulators of the plain path (3 per corner)
-    DevBuf<double> d_x0c, d_keys, d_fit;
+    DevBuf<double> d_fit, d_fit_part;
+    DevBuf<int> d_fit_arrived;
     DevBuf<float2> d_sc;
     DevBuf<unsigned char> d_pe;
     DevBuf<float> d_compact;
@@ -327,6 +335,7 @@ extern "C" {
 static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subset = nullptr);
 static sim_status build_packed_items(voxsim_ctx* ctx, const std::vector<std::vector<std::pair<int, int>>>& lattice,
                                      const std::vector<int>& mass_groups, bool damped);
+static sim_status run_topology(voxsim_ctx* ctx, bool packed);
 }
 
 namespace {
@@ -374,12 +383,6 @@ sim_status status_from_words(const int32_t* w)
         return fail(SIM_ETIMEOUT, "topology: the component labelling hit its iteration bound");
     if (w[0] & 2) return fail(SIM_EINVAL, "material id out of range 0..4 in device genomes");
     return SIM_OK;
-}
-
-__global__ void k_spring_keys(const int* ns, int P, double* keys)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < P) keys[i] = (double)ns[i];
 }
 
 }  // namespace
@@ -500,18 +503,23 @@ sim_status sim_set_population(voxsim_ctx* ctx, int32_t P, const int32_t* dims, i
     VX_CK(ctx->d_dims.ensure(3 * (size_t)P));
     VX_CK(ctx->d_voff.ensure(P + 1)); VX_CK(ctx->d_moff.ensure(P + 1)); VX_CK(ctx->d_soff.ensure(P + 1));
     VX_CK(ctx->d_tmp_off.ensure(P + 1));
-    VX_CK(ctx->d_nm.ensure(P)); VX_CK(ctx->d_ns.ensure(P)); VX_CK(ctx->d_lpt.ensure(P));
+    VX_CK(ctx->d_nm.ensure(P)); VX_CK(ctx->d_ns.ensure(P));
     VX_CK(ctx->d_queue.ensure(2)); VX_CK(ctx->d_status.ensure(4));
     VX_CK(ctx->d_mat_raw.ensure(V)); VX_CK(ctx->d_mat.ensure(V));
     VX_CK(ctx->d_w.ensure(V)); VX_CK(ctx->d_kappa.ensure(V)); VX_CK(ctx->d_phi.ensure(V));
-    VX_CK(ctx->d_label.ensure(V)); VX_CK(ctx->d_count.ensure(V));
-    VX_CK(ctx->d_corner_mass.ensure(Mc)); VX_CK(ctx->d_mass_corner.ensure(Mc));
+    VX_CK(ctx->d_vox_q.ensure(V)); VX_CK(ctx->d_vox_s.ensure(V));
+    VX_CK(ctx->d_corner_mass.ensure(Mc)); VX_CK(ctx->d_corner_spring.ensure(Mc)); VX_CK(ctx->d_mass_corner.ensure(Mc));
     VX_CK(ctx->d_sab.ensure(Sc)); VX_CK(ctx->d_sp.ensure(Sc));
     if (packed) VX_CK(ctx->d_spack.ensure(Sc));
     ctx->have_pack = packed;
     VX_CK(ctx->d_x0.ensure(Mc)); VX_CK(ctx->d_x.ensure(Mc)); VX_CK(ctx->d_v.ensure(Mc));
     VX_CK(ctx->d_cflags.ensure(Mc)); VX_CK(ctx->d_prm.ensure(39 * (size_t)Mc));
-    VX_CK(ctx->d_x0c.ensure(P)); VX_CK(ctx->d_keys.ensure(P)); VX_CK(ctx->d_fit.ensure(P));
+    VX_CK(ctx->d_fit.ensure(P));
+    if (fitness_chunks(max_corner) > 1) {
+        VX_CK(ctx->d_fit_part.ensure((size_t)P * fitness_chunks(max_corner)));
+        VX_CK(ctx->d_fit_arrived.ensure(P));
+        VX_CK(cudaMemsetAsync(ctx->d_fit_arrived.p, 0, sizeof(int) * P, s));
+    }
     ctx->dims = d; ctx->voff = voff; ctx->moff = moff; ctx->soff = soff;
     ctx->P = P; ctx->V_tot = V; ctx->M_cap = Mc; ctx->S_cap = Sc;
     ctx->max_corner = max_corner; ctx->max_spring_cap = max_sc;
@@ -604,16 +612,7 @@ sim_status sim_set_population(voxsim_ctx* ctx, int32_t P, const int32_t* dims, i
                                                 ctx->num_sms, s));
         }
         // topology
-        VX_LAUNCH(ctx, launch_topology(ctx->view(), ctx->d_mat_raw.p, ctx->d_mat.p, ctx->d_w.p, ctx->d_kappa.p,
-                              ctx->d_phi.p, mc, ctx->p.edge, ctx->d_label.p, ctx->d_count.p,
-                              ctx->d_corner_mass.p, ctx->d_mass_corner.p, ctx->d_sab.p, ctx->d_sp.p,
-                              packed ? ctx->d_spack.p : nullptr, ctx->d_cflags.p, ctx->d_prm.p,
-                              ctx->d_x0.p, ctx->d_x.p, ctx->d_v.p,
-                              ctx->d_x0c.p, ctx->d_status.p, 0, s));
-        // longest-first processing order (by spring count, ties by index)
-        k_spring_keys<<<(P + 255) / 256, 256, 0, s>>>(ctx->d_ns.p, P, ctx->d_keys.p);
-        VX_LAUNCH(ctx, cudaGetLastError());
-        VX_LAUNCH(ctx, launch_evo_rank(ctx->d_keys.p, P, ctx->d_lpt.p, s));
+        if (sim_status st = run_topology(ctx, packed)) return st;
         // the mass counts order the work queue (longest first); the plan is built on the host
         ctx->mass_count.assign(P, 0);
         ctx->spring_count.assign(P, 0);
@@ -629,6 +628,73 @@ sim_status sim_set_population(voxsim_ctx* ctx, int32_t P, const int32_t* dims, i
     ctx->rec_valid = false;
     ctx->drop_graph();
     ctx->have_pop = true;
+    return SIM_OK;
+}
+
+// Components, masses, springs, tables and initial state of the decoded population: one launch for
+// the robots of at most topology_small_corners() corners, a few for the larger ones.
+static sim_status run_topology(voxsim_ctx* ctx, bool packed)
+{
+    cudaStream_t s = ctx->stream;
+    const int P = ctx->P;
+    std::vector<int> small, large;
+    int vox[2] = {0, 0}, cor[2] = {0, 0};                // largest voxel and corner counts: small, large
+    for (int r = 0; r < P; ++r) {
+        const int C = (int)(ctx->moff[r + 1] - ctx->moff[r]), V = (int)(ctx->voff[r + 1] - ctx->voff[r]);
+        const int k = C <= topology_small_corners() ? 0 : 1;
+        (k ? large : small).push_back(r);
+        vox[k] = std::max(vox[k], V);
+        cor[k] = std::max(cor[k], C);
+    }
+    TopoArgs a{};
+    a.pv = ctx->view();
+    a.mat_raw = ctx->d_mat_raw.p;
+    a.w = ctx->d_w.p;
+    a.kappa = ctx->d_kappa.p;
+    a.phi = ctx->d_phi.p;
+    a.mat = ctx->d_mat.p;
+    a.vox_q = ctx->d_vox_q.p;
+    a.vox_s = ctx->d_vox_s.p;
+    a.corner_mass = ctx->d_corner_mass.p;
+    a.corner_spring = ctx->d_corner_spring.p;
+    a.mass_corner = ctx->d_mass_corner.p;
+    a.spr_ab = ctx->d_sab.p;
+    a.spr_p = ctx->d_sp.p;
+    a.spr_pack = packed ? ctx->d_spack.p : nullptr;
+    a.cflags = ctx->d_cflags.p;
+    a.prm = ctx->d_prm.p;
+    a.x0 = ctx->d_x0.p;
+    a.x = ctx->d_x.p;
+    a.v = ctx->d_v.p;
+    a.mc = ctx->matconst();
+    a.edge = ctx->p.edge;
+    a.rest1 = (float)ctx->p.edge;
+    a.rest2 = (float)(ctx->p.edge * 1.4142135623730951);
+    a.rest3 = (float)(ctx->p.edge * 1.7320508075688772);
+    if (!large.empty()) {
+        // (the host copy lives in the context: the upload may still read it after this call)
+        ctx->topo_robots = small;
+        ctx->topo_robots.insert(ctx->topo_robots.end(), large.begin(), large.end());
+        VX_CK(ctx->d_topo_robots.ensure(P));
+        VX_CK(ctx->d_label.ensure(ctx->V_tot)); VX_CK(ctx->d_count.ensure(ctx->V_tot));
+        VX_CK(ctx->d_best.ensure(P)); VX_CK(ctx->d_zmin.ensure(P));
+        VX_CK(ctx->d_chunk.ensure(topology_chunks(cor[1]) * std::min<size_t>(large.size(), 32768)));
+        VX_CK(cudaMemcpyAsync(ctx->d_topo_robots.p, ctx->topo_robots.data(), sizeof(int) * P, cudaMemcpyHostToDevice, s));
+        a.label = ctx->d_label.p;
+        a.count = ctx->d_count.p;
+        a.best = ctx->d_best.p;
+        a.zmin = ctx->d_zmin.p;
+        a.chunk = ctx->d_chunk.p;
+        const size_t slice = 32768;                      // robots per launch (grid.y)
+        for (size_t i = 0; i < large.size(); i += slice) {
+            a.robots = ctx->d_topo_robots.p + small.size() + i;
+            int n = 0;
+            VX_LAUNCH(ctx, launch_topology_large(a, (int)std::min(slice, large.size() - i), vox[1], cor[1], s, &n));
+            ctx->launches += n - 1;
+        }
+        a.robots = ctx->d_topo_robots.p;
+    }
+    if (!small.empty()) VX_LAUNCH(ctx, launch_topology_small(a, (int)small.size(), vox[0], cor[0], ctx->num_sms, s));
     return SIM_OK;
 }
 
@@ -1345,7 +1411,8 @@ sim_status sim_fitness(voxsim_ctx* ctx, double* out, int32_t mem)
     cudaStream_t s = ctx->stream;
     double* dst = mem == SIM_MEM_DEVICE ? out : ctx->d_fit.p;
     VX_LAUNCH(ctx, launch_fitness(ctx->view(), ctx->d_mass_corner.p, ctx->d_x.p, ctx->d_x0.p,
-                                  (float)ctx->p.dead_bound, dst, s));
+                                  (float)ctx->p.dead_bound, fitness_chunks(ctx->max_corner), ctx->d_fit_part.p,
+                                  ctx->d_fit_arrived.p, dst, s));
     if (mem == SIM_MEM_HOST) {
         // the status words ride along: a segmented lattice step that gave up waiting shows here
         int32_t words[4];

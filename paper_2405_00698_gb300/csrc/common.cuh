@@ -111,12 +111,41 @@ cudaError_t launch_mlp_query_simt(int P, int Q, const void* pe_bf16, const float
                                   MatConst mc, uint8_t* mat, float* w, float* kappa, float* phi,
                                   cudaStream_t s);
 
-cudaError_t launch_topology(PopView pv, const uint8_t* mat_raw, uint8_t* mat, const float* w,
-                            const float* kappa, const float* phi, MatConst mc, double edge,
-                            int* label, int* count, int* corner_mass, int* mass_corner,
-                            int2* spr_ab, float4* spr_p, float4* spr_pack, uint32_t* cflags,
-                            float* prm, float4* x0, float4* x, float4* v, double* x0c, int* status,
-                            int max_threads, cudaStream_t s);
+// Components, masses, springs, lattice tables and initial state (see topology.cu).
+struct TopoArgs {
+    PopView pv;
+    const int* robots;       // the robots of the launch (NULL for the small ones: all, in order)
+    const uint8_t* mat_raw;  // per voxel: decoded material, weight, stiffness, phase
+    const float* w;
+    const float* kappa;
+    const float* phi;
+    uint8_t* mat;            // per voxel: material kept (0 outside the largest component)
+    float4* vox_q;           // scratch per voxel: (w, kappa, amplitude, cos phi), sin phi
+    float* vox_s;
+    int* label;              // scratch per voxel and totals per robot (large robots)
+    int* count;
+    unsigned long long* best;
+    int* zmin;
+    int2* chunk;             // masses and springs per corner chunk
+    int* corner_mass;        // per corner: mass index or -1; where its springs start in the list
+    int* corner_spring;
+    int* mass_corner;        // per robot at moff: corners of the masses, ascending
+    int2* spr_ab;            // spring list
+    float4* spr_p;
+    float4* spr_pack;        // direction-major packed springs (NULL: not wanted)
+    uint32_t* cflags;
+    float* prm;
+    float4* x0;
+    float4* x;
+    float4* v;
+    MatConst mc;
+    double edge;
+    float rest1, rest2, rest3;   // rest lengths of the edge, face and body diagonals
+};
+int topology_small_corners();            // robots of at most so many corners take the small launch
+size_t topology_chunks(int max_corners); // entries of `chunk` per large robot
+cudaError_t launch_topology_small(const TopoArgs& a, int n, int max_vox, int max_corners, int num_sms, cudaStream_t s);
+cudaError_t launch_topology_large(const TopoArgs& a, int n, int max_vox, int max_corners, cudaStream_t s, int* launches);
 
 cudaError_t launch_sincos_table(double omega, double dt, int64_t step0, int n, float2* out,
                                 cudaStream_t s);
@@ -325,8 +354,11 @@ cudaError_t launch_step_roles(const LatticeArgs& a, int max_corners, cudaStream_
 cudaError_t launch_step_lattice_packed(const LatticeArgs& a, int grid, size_t smem, cudaStream_t s);
 size_t resident_smem_bytes(int max_mass, int max_spring_smem, int accumulate);
 
+// chunks = fitness_chunks(largest robot's corners); with more than one, partial holds P x chunks sums
+// and arrived P counters (zero before the first call; the kernel leaves them zero).
+int fitness_chunks(int max_corners);
 cudaError_t launch_fitness(PopView pv, const int* mass_corner, const float4* u, const float4* x0,
-                           float dead_bound, double* out, cudaStream_t s);
+                           float dead_bound, int chunks, double* partial, int* arrived, double* out, cudaStream_t s);
 
 cudaError_t launch_evo_rank(const double* fitness, int P, int* order, cudaStream_t s);
 cudaError_t launch_elite_weights(const int* order, const double* fitness, int P, int E, double* w,
