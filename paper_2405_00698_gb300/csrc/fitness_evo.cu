@@ -83,24 +83,10 @@ k_fitness(PopView pv, const int* __restrict__ mass_corner, const float4* __restr
 // number `ctr` of the stream seeded with `seed` is the SplitMix64 finaliser applied to
 // seed + (ctr + 1) * golden-gamma.
 // ----------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint64_t ctr)
-{
-    uint64_t z = seed + (ctr + 1ull) * 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-
 enum { kParentA = 0, kParentB = 1, kMask = 2, kMutate = 3, kU1 = 4, kU2 = 5, kCross = 6 };
 
-// High 32 bits of the draw for (generation, child, gene, purpose), fields packed as
-// generation | child (16 bits) | gene (26 bits) | purpose (3 bits).
-__device__ __forceinline__ uint32_t draw32(uint64_t seed, uint64_t gen, uint32_t child,
-                                           uint32_t gene, uint32_t purpose)
-{
-    const uint64_t ctr = ((((gen << 16) | child) << 26 | gene) << 3) | purpose;
-    return (uint32_t)(splitmix64_at(seed, ctr) >> 32);
-}
+// A draw is the high 32 bits of the output for (generation, child, gene, purpose), fields packed as
+// generation | child (16 bits) | gene (26 bits) | purpose (3 bits): see row_draw.
 
 // Rank by counting: the rank of robot i is the number of robots ordered before it
 // (larger fitness, or equal fitness and smaller index; NaN counts as -infinity).  The fitness
@@ -115,40 +101,87 @@ __device__ __forceinline__ unsigned long long rank_key(double x)
     return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
 }
 
-__global__ void k_rank(const double* __restrict__ f, int P, int* __restrict__ order)
+// A warp ranks kRankPer robots: its lanes share the comparisons with all others, tile by tile from
+// shared memory, so 1024 robots spread over 32 blocks (one thread per robot, as before, left all but
+// 4 SMs idle: 17 us; now 6.7).
+constexpr int kRankThreads = 256;
+constexpr int kRankPer = 4;
+
+__global__ void __launch_bounds__(kRankThreads) k_rank(const double* __restrict__ f, int P, int* __restrict__ order)
 {
-    extern __shared__ unsigned long long tile[];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const unsigned long long ki = i < P ? rank_key(f[i]) : 0ull;
-    int rank = 0;
-    for (int base = 0; base < P; base += blockDim.x) {
+    __shared__ unsigned long long tile[kRankThreads];
+    const int lane = threadIdx.x & 31;
+    const int i0 = (blockIdx.x * (kRankThreads / 32) + (threadIdx.x >> 5)) * kRankPer;
+    unsigned long long key[kRankPer];
+    int rank[kRankPer];
+#pragma unroll
+    for (int k = 0; k < kRankPer; ++k) {
+        key[k] = i0 + k < P ? rank_key(f[i0 + k]) : ~0ull;
+        rank[k] = 0;
+    }
+    for (int base = 0; base < P; base += kRankThreads) {
         __syncthreads();
         const int j = base + threadIdx.x;
-        tile[threadIdx.x] = j < P ? rank_key(f[j]) : 0ull;
+        tile[threadIdx.x] = j < P ? rank_key(f[j]) : 0ull;   // (0: before no robot, see below)
         __syncthreads();
-        const int n = min((int)blockDim.x, P - base);
-        if (i < P)
-            for (int t = 0; t < n; ++t) {
-                const unsigned long long kg = tile[t];
-                const int jj = base + t;
-                rank += (kg > ki) || (kg == ki && jj < i);
-            }
+#pragma unroll
+        for (int t = lane; t < kRankThreads; t += 32) {
+            const unsigned long long kg = tile[t];
+            const int jj = base + t;
+#pragma unroll
+            for (int k = 0; k < kRankPer; ++k) rank[k] += (kg > key[k]) || (kg == key[k] && jj < i0 + k);
+        }
     }
-    if (i < P) order[rank] = i;
+    // entries past P have key 0, below every robot's (the least is that of -infinity), so they count
+    // for none
+#pragma unroll
+    for (int k = 0; k < kRankPer; ++k) {
+        for (int o = 16; o > 0; o >>= 1) rank[k] += __shfl_xor_sync(0xffffffffu, rank[k], o);
+        if (lane == 0 && i0 + k < P) order[rank[k]] = i0 + k;
+    }
 }
 
-// One thread per (child row, gene).  Elite rows copy their genome; child rows pick parents,
-// crossover mask and mutation from the counter-based generator.
-__global__ void k_children(const float* __restrict__ gin, float* __restrict__ gout,
-                           const int* __restrict__ order, int P, int G, int E, uint64_t seed,
-                           uint64_t gen, uint32_t thresh, float sigma, uint32_t keep,
-                           int* __restrict__ parents, uint8_t* __restrict__ mask)
+// Draw number `purpose` of gene j of a row whose counters start at `ctr0` (generation and child
+// packed above gene and purpose): z = seed + (ctr + 1) gamma with the row's part added up before.
+__device__ __forceinline__ uint32_t row_draw(uint64_t z0, uint32_t j, uint32_t purpose)
 {
-    const int c = blockIdx.y;
+    constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ull;
+    uint64_t z = z0 + (uint64_t)j * (8ull * kGamma) + purpose * kGamma;
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return (uint32_t)((z ^ (z >> 31)) >> 32);
+}
+
+// A block takes kChildGenes genes of a row.  Elite rows copy their genome; child rows pick parents,
+// crossover mask and mutation from the counter-based generator.  A gene mutates with probability
+// 0.1 or so, so nearly every warp holds a mutating lane: the warp queues its mutating genes in
+// shared memory and evaluates the Gaussian for 32 of them at a time instead of for each warp of 32
+// genes (1024 genomes of 20,998 genes: 152 -> 78 us; 107 MB through device memory, 16 us; the
+// generator's 64-bit products are what is left).
+constexpr int kChildThreads = 256;
+constexpr int kChildGenes = 8 * kChildThreads;
+
+__device__ __forceinline__ float mutated(uint64_t z0, uint32_t j, float g, float sigma)
+{
+    const float u1 = ((float)row_draw(z0, j, kU1) + 1.0f) * 2.3283064365386963e-10f;
+    const float u2 = (float)row_draw(z0, j, kU2) * 2.3283064365386963e-10f;
+    const float z = sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
+    return g + sigma * z;
+}
+
+__global__ void __launch_bounds__(kChildThreads)
+k_children(const float* __restrict__ gin, float* __restrict__ gout, const int* __restrict__ order, int P, int G,
+           int E, uint64_t seed, uint64_t gen, uint32_t thresh, float sigma, uint32_t keep,
+           int* __restrict__ parents, uint8_t* __restrict__ mask)
+{
+    __shared__ uint32_t sh_j[kChildThreads / 32][64];
+    __shared__ float sh_g[kChildThreads / 32][64];
+    const int c = blockIdx.y, j0 = blockIdx.x * kChildGenes, j1 = min(G, j0 + kChildGenes);
     const size_t row = (size_t)c * G;
     if (c < E) {
         const float* src = gin + (size_t)order[c] * G;
-        for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < G; j += gridDim.x * blockDim.x) {
+#pragma unroll 8
+        for (int j = j0 + threadIdx.x; j < j1; j += kChildThreads) {
             gout[row + j] = src[j];
             if (mask) mask[row + j] = 0;
         }
@@ -158,8 +191,9 @@ __global__ void k_children(const float* __restrict__ gin, float* __restrict__ go
         }
         return;
     }
-    const uint32_t ua = draw32(seed, gen, c, 0, kParentA);
-    const uint32_t ub = draw32(seed, gen, c, 0, kParentB);
+    const uint64_t z0 = seed + (((((gen << 16) | (uint64_t)c) << 26) << 3) + 1ull) * 0x9E3779B97F4A7C15ull;
+    const uint32_t ua = row_draw(z0, 0, kParentA);
+    const uint32_t ub = row_draw(z0, 0, kParentB);
     const int pa = order[(int)(((uint64_t)ua * (uint64_t)E) >> 32)];
     const int pb = order[(int)(((uint64_t)ub * (uint64_t)E) >> 32)];
     if (parents && blockIdx.x == 0 && threadIdx.x == 0) {
@@ -169,19 +203,38 @@ __global__ void k_children(const float* __restrict__ gin, float* __restrict__ go
     const float* A = gin + (size_t)pa * G;
     const float* Bp = gin + (size_t)pb * G;
     // crossover rate below 1: some children copy parent A (a draw per child)
-    const bool copy_a = keep != 0u && draw32(seed, gen, c, 0, kCross) < keep;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < G; j += gridDim.x * blockDim.x) {
-        const uint32_t m = copy_a ? 1u : draw32(seed, gen, c, j, kMask) >> 31;
-        float g = m ? A[j] : Bp[j];
-        if (draw32(seed, gen, c, j, kMutate) < thresh) {
-            const float u1 = ((float)draw32(seed, gen, c, j, kU1) + 1.0f) * 2.3283064365386963e-10f;
-            const float u2 = (float)draw32(seed, gen, c, j, kU2) * 2.3283064365386963e-10f;
-            const float z = sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
-            g = g + sigma * z;
+    const bool copy_a = keep != 0u && row_draw(z0, 0, kCross) < keep;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t* qj = sh_j[warp];
+    float* qg = sh_g[warp];
+    int queued = 0;                                       // of the warp, below 32 between rounds
+    for (int jb = j0 + 32 * warp; jb < j1; jb += kChildThreads) {
+        const int j = jb + lane;
+        bool mut = false;
+        float g = 0.f;
+        if (j < j1) {
+            const uint32_t m = copy_a ? 1u : row_draw(z0, j, kMask) >> 31;
+            g = m ? A[j] : Bp[j];
+            mut = row_draw(z0, j, kMutate) < thresh;
+            if (!mut) gout[row + j] = g;
+            if (mask) mask[row + j] = (uint8_t)m;
         }
-        gout[row + j] = g;
-        if (mask) mask[row + j] = (uint8_t)m;
+        const unsigned w = __ballot_sync(0xffffffffu, mut);
+        if (mut) {
+            const int at = queued + __popc(w & ((1u << lane) - 1u));
+            qj[at] = (uint32_t)j;
+            qg[at] = g;
+        }
+        queued += __popc(w);
+        __syncwarp();
+        if (queued >= 32) {
+            queued -= 32;                                 // the last 32 of the queue
+            const uint32_t jm = qj[queued + lane];
+            gout[row + jm] = mutated(z0, jm, qg[queued + lane], sigma);
+            __syncwarp();
+        }
     }
+    if (lane < queued) gout[row + qj[lane]] = mutated(z0, qj[lane], qg[lane], sigma);
 }
 
 // sin and cos of w t for the steps of one call, FP64 then rounded to float:
@@ -254,8 +307,8 @@ cudaError_t launch_elite_weights(const int* order, const double* fitness, int P,
 
 cudaError_t launch_evo_rank(const double* fitness, int P, int* order, cudaStream_t s)
 {
-    const int T = 256;
-    k_rank<<<(P + T - 1) / T, T, T * sizeof(unsigned long long), s>>>(fitness, P, order);
+    constexpr int per_block = kRankThreads / 32 * kRankPer;
+    k_rank<<<(P + per_block - 1) / per_block, kRankThreads, 0, s>>>(fitness, P, order);
     return cudaGetLastError();
 }
 
@@ -263,11 +316,8 @@ cudaError_t launch_evo_children(const float* gin, float* gout, const int* order,
                                 int E, uint64_t seed, uint64_t gen, uint32_t thresh, float sigma,
                                 uint32_t keep, int* parents, uint8_t* mask, cudaStream_t s)
 {
-    const int T = 256;
-    int bx = (G + T - 1) / T;
-    if (bx > 64) bx = 64;
-    dim3 grid(bx, P);
-    k_children<<<grid, T, 0, s>>>(gin, gout, order, P, G, E, seed, gen, thresh, sigma, keep, parents,
+    const dim3 grid((G + kChildGenes - 1) / kChildGenes, P);
+    k_children<<<grid, kChildThreads, 0, s>>>(gin, gout, order, P, G, E, seed, gen, thresh, sigma, keep, parents,
                                   mask);
     return cudaGetLastError();
 }
@@ -296,39 +346,75 @@ cudaError_t launch_compact_state(PopView pv, const int* mass_corner, const float
 //           mean_{i != j} |g_i - g_j|^2 = 2 P / (P - 1) * mean_i |g_i - mean g|^2;
 //   morphology: mean over robot pairs of the fraction of voxels whose kept materials differ,
 //           from per-voxel material counts c_k: differing pairs = (P^2 - sum_k c_k^2) / 2.
-// FP64 accumulation; one block per gene / voxel chunk, atomics into two FP64 totals.
+// FP64 accumulation, atomics into two FP64 totals.
 // ----------------------------------------------------------------------------------------------
 namespace vx {
 namespace {
 
-__global__ void k_genome_spread(const float* __restrict__ g, int P, int G, double* __restrict__ total)
+// A block takes kSpreadCols genes (or voxels), its thread rows share the population's rows; before,
+// a thread took a whole column and most SMs stood empty (1024 genomes of
+// 20,998 genes: 250 -> 142 us; 1024 robots 8x8x8: 412 -> 10 us).
+constexpr int kSpreadCols = 32;
+constexpr int kSpreadRows = 8;       // (the FP64 units bound it; 32 rows: 171 us)
+constexpr int kMorphRows = 32;       // (8: 23 us)
+
+__global__ void __launch_bounds__(kSpreadCols * kSpreadRows)
+k_genome_spread(const float* __restrict__ g, int P, int G, double* __restrict__ total)
 {
-    double acc = 0.0;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < G; j += gridDim.x * blockDim.x) {
-        double s = 0.0, s2 = 0.0;
-        for (int i = 0; i < P; ++i) {
-            const double x = (double)g[(size_t)i * G + j];
-            s += x;
-            s2 += x * x;
+    __shared__ double sh[2][kSpreadRows][kSpreadCols];
+    const int x = threadIdx.x, y = threadIdx.y, j = blockIdx.x * kSpreadCols + x;
+    double s = 0.0, s2 = 0.0;
+    if (j < G) {
+#pragma unroll 8
+        for (int i = y; i < P; i += kSpreadRows) {
+            const double v = (double)g[(size_t)i * G + j];
+            s += v;
+            s2 += v * v;
         }
-        acc += s2 - s * s / P;             // sum_i (g_ij - mean_j)^2
     }
+    sh[0][y][x] = s;
+    sh[1][y][x] = s2;
+    __syncthreads();
+    if (y != 0) return;
+#pragma unroll
+    for (int i = 1; i < kSpreadRows; ++i) {
+        s += sh[0][i][x];
+        s2 += sh[1][i][x];
+    }
+    double acc = s2 - s * s / P;                           // sum_i (g_ij - mean_j)^2 (0 past the last gene)
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(total, acc);
+    if (x == 0) atomicAdd(total, acc);
 }
 
-__global__ void k_morph_spread(const uint8_t* __restrict__ mat, int P, int V, double* __restrict__ total)
+__global__ void __launch_bounds__(kSpreadCols * kMorphRows)
+k_morph_spread(const uint8_t* __restrict__ mat, int P, int V, double* __restrict__ total)
 {
+    __shared__ int sh_c[kSpreadCols][kNumMat];
+    const int x = threadIdx.x, y = threadIdx.y, v = blockIdx.x * kSpreadCols + x;
+    if (y < kNumMat) sh_c[x][y] = 0;
+    __syncthreads();
+    int c[kNumMat] = {0, 0, 0, 0, 0};
+    if (v < V) {
+#pragma unroll 4
+        for (int i = y; i < P; i += kMorphRows) {
+            const int m = mat[(size_t)i * V + v] % kNumMat;
+#pragma unroll
+            for (int k = 0; k < kNumMat; ++k) c[k] += m == k;
+        }
+#pragma unroll
+        for (int k = 0; k < kNumMat; ++k)
+            if (c[k]) atomicAdd(&sh_c[x][k], c[k]);
+    }
+    __syncthreads();
+    if (y != 0) return;
     double acc = 0.0;
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
-        int c[kNumMat] = {0, 0, 0, 0, 0};
-        for (int i = 0; i < P; ++i) c[mat[(size_t)i * V + v] % kNumMat]++;
+    if (v < V) {
         double eq = 0.0;
-        for (int k = 0; k < kNumMat; ++k) eq += (double)c[k] * c[k];
-        acc += ((double)P * P - eq) * 0.5;  // pairs of robots that differ at voxel v
+        for (int k = 0; k < kNumMat; ++k) eq += (double)sh_c[x][k] * sh_c[x][k];
+        acc = ((double)P * P - eq) * 0.5;                  // pairs of robots that differ at voxel v
     }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(total, acc);
+    if (x == 0) atomicAdd(total, acc);
 }
 
 }  // namespace
@@ -338,8 +424,10 @@ cudaError_t launch_diversity(const float* genomes, int P, int G, const uint8_t* 
 {
     cudaError_t e = cudaMemsetAsync(totals, 0, 2 * sizeof(double), s);
     if (e != cudaSuccess) return e;
-    if (genomes && G > 0) k_genome_spread<<<std::min((G + 255) / 256, 1024), 256, 0, s>>>(genomes, P, G, totals);
-    if (mat && V > 0) k_morph_spread<<<std::min((V + 255) / 256, 1024), 256, 0, s>>>(mat, P, V, totals + 1);
+    const dim3 block(kSpreadCols, kSpreadRows);
+    if (genomes && G > 0) k_genome_spread<<<(G + kSpreadCols - 1) / kSpreadCols, block, 0, s>>>(genomes, P, G, totals);
+    if (mat && V > 0)
+        k_morph_spread<<<(V + kSpreadCols - 1) / kSpreadCols, dim3(kSpreadCols, kMorphRows), 0, s>>>(mat, P, V, totals + 1);
     return cudaGetLastError();
 }
 
