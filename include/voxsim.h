@@ -59,7 +59,8 @@ enum {
 
 /* Force accumulation of the time stepping kernels. */
 enum {
-    SIM_ACC_AUTO = 0,   /* library choice (measured default) */
+    SIM_ACC_AUTO = 0,   /* library choice (measured default): a fixed order wherever a robot's force rows
+                           fit shared memory, shared-memory atomics for larger or damped ones */
     SIM_ACC_ATOMIC = 1, /* per-spring threads add into per-mass accumulators atomically */
     SIM_ACC_GATHER = 2  /* every mass sums its springs' forces in a fixed order (lattice-gather
                            kernel, a cluster of lattice blocks for robots of up to 8 x 768

@@ -186,6 +186,10 @@ struct voxsim_ctx {
     // atomic-kernel groups (one persistent launch each): robots of one thread count
     struct AtomicGroup { int threads; int first; int count; int max_corner; int64_t max_spring_cap; };
     std::vector<AtomicGroup> atomic_groups;
+    // robots on the per-mass kernel of 1024-thread blocks (step_rows.cu): one persistent launch
+    std::vector<int> rows_robots;
+    int rows_max_corner = 0, rows_max_mass = 0, rows_nd = 0;
+    DevBuf<int> d_rows;
     // cluster lattice groups (one launch each): robots cut into q slabs
     struct ClusterGroup { int q; int first; int count; };
     std::vector<ClusterGroup> cluster_groups;
@@ -504,7 +508,7 @@ sim_status sim_set_population(voxsim_ctx* ctx, int32_t P, const int32_t* dims, i
     VX_CK(ctx->d_voff.ensure(P + 1)); VX_CK(ctx->d_moff.ensure(P + 1)); VX_CK(ctx->d_soff.ensure(P + 1));
     VX_CK(ctx->d_tmp_off.ensure(P + 1));
     VX_CK(ctx->d_nm.ensure(P)); VX_CK(ctx->d_ns.ensure(P));
-    VX_CK(ctx->d_queue.ensure(2)); VX_CK(ctx->d_status.ensure(4));
+    VX_CK(ctx->d_queue.ensure(3)); VX_CK(ctx->d_status.ensure(4));
     VX_CK(ctx->d_mat_raw.ensure(V)); VX_CK(ctx->d_mat.ensure(V));
     VX_CK(ctx->d_w.ensure(V)); VX_CK(ctx->d_kappa.ensure(V)); VX_CK(ctx->d_phi.ensure(V));
     VX_CK(ctx->d_vox_q.ensure(V)); VX_CK(ctx->d_vox_s.ensure(V));
@@ -763,6 +767,7 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
     ctx->atomic_groups.clear();
     if (ctx->p.path == SIM_PATH_PLAIN) {       // every robot on the baseline kernels
         ctx->n_items = ctx->n_items_corner = ctx->n_big = ctx->n_stream = ctx->n_cluster = 0;
+        ctx->rows_robots.clear();
         ctx->cluster_groups.clear();
         VX_CK(ctx->d_plain_f.ensure(3 * (size_t)ctx->M_cap));
         VX_CK(cudaMemsetAsync(ctx->d_plain_f.p, 0, sizeof(float) * 3 * (size_t)ctx->M_cap, ctx->stream));
@@ -772,6 +777,7 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
     const bool damped = ctx->stepconst().damped != 0;
     std::vector<std::vector<std::pair<int, int>>> lattice(6), lattice_sp(6);
     std::vector<std::pair<int, std::pair<int, int>>> atomic;   // (threads, (-corners, robot))
+    std::vector<std::pair<int, int>> rows;                       // (-masses, robot), of the atomic ones
     std::vector<int> streamed;
     std::vector<std::pair<int, int>> clustered;                  // (q, robot)
     std::vector<int> mass_groups;                                // larger robots in mass-sized groups
@@ -849,6 +855,10 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
             // longest first: by spring count when known (a thread per spring), else corners
             const int key = (int)ctx->spring_count.size() == ctx->P ? ctx->spring_count[r] : C;
             atomic.push_back({threads, {-key, r}});
+            // no block size was asked for or tuned: the per-mass kernel where its rows fit (below)
+            if (ctx->p.accumulate == SIM_ACC_AUTO && ctx->p.threads <= 0 && ctx->class_threads[k] <= 0 && !damped &&
+                (int)ctx->mass_count.size() == ctx->P && rows_per_corner(C, budget) > 0)
+                rows.push_back({-ctx->mass_count[r], r});
         } else {
             streamed.push_back(r);
             ctx->max_stream_corner = std::max(ctx->max_stream_corner, C);
@@ -902,6 +912,27 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
         ctx->roles_max_corner = corners;
     }
     if (sim_status st = build_packed_items(ctx, lattice, mass_groups, damped)) return st;
+    // The per-mass kernel (step_rows.cu) takes every robot of the atomic kernel that it can, unless
+    // that would leave two launches that each fill only part of the SMs (20 robots 12x12x12 of 1884 to
+    // 2081 masses, split at 2048: 4.4 ms in two launches, 2.6 ms in one).  Undamped robots only:
+    // with dashpots its square roots cost more than the atomics they replace (100 robots 10x10x10,
+    // 200 steps: 2.17 ms on the atomic kernel, 2.44 on this one).
+    if (rows.size() < atomic.size() && (int)rows.size() < ctx->num_sms) rows.clear();
+    std::sort(rows.begin(), rows.end());               // longest first
+    ctx->rows_robots.clear();
+    ctx->rows_max_corner = 0;
+    ctx->rows_max_mass = rows.empty() ? 0 : -rows[0].first;
+    std::vector<char> in_rows(rows.empty() ? 0 : ctx->P, 0);
+    for (const auto& q : rows) {
+        ctx->rows_robots.push_back(q.second);
+        in_rows[q.second] = 1;
+        ctx->rows_max_corner = std::max(ctx->rows_max_corner, (int)(ctx->moff[q.second + 1] - ctx->moff[q.second]));
+    }
+    ctx->rows_nd = rows.empty() ? 0 : rows_per_corner(ctx->rows_max_corner, budget);
+    if (!rows.empty())
+        atomic.erase(std::remove_if(atomic.begin(), atomic.end(),
+                                    [&](const std::pair<int, std::pair<int, int>>& q) { return in_rows[q.second.second] != 0; }),
+                     atomic.end());
     std::sort(atomic.begin(), atomic.end());
     std::vector<int> big;
     for (size_t i = 0; i < atomic.size();) {
@@ -937,7 +968,10 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
         ctx->stream_cube40 = ctx->stream_cube40 && ctx->dims[3 * r] == 40 && ctx->dims[3 * r + 1] == 40 &&
                              ctx->dims[3 * r + 2] == 40;
     cudaStream_t s = ctx->stream;
-    VX_CK(ctx->d_queue.ensure(2 + ctx->atomic_groups.size()));
+    VX_CK(ctx->d_queue.ensure(3 + ctx->atomic_groups.size()));
+    VX_CK(ctx->d_rows.ensure(rows.size()));
+    if (!rows.empty())
+        VX_CK(cudaMemcpyAsync(ctx->d_rows.p, ctx->rows_robots.data(), sizeof(int) * rows.size(), cudaMemcpyHostToDevice, s));
     if (!streamed.empty()) {
         VX_CK(ctx->d_stream.ensure(streamed.size()));
         VX_CK(cudaMemcpyAsync(ctx->d_stream.p, streamed.data(), sizeof(int) * streamed.size(),
@@ -1204,10 +1238,30 @@ static sim_status step_cluster(voxsim_ctx* ctx, int n)
     return SIM_OK;
 }
 
-// The atomic resident kernel: one persistent launch per thread count.
+// The robots of more than a block's corners and masses: the per-mass kernel of 1024-thread blocks,
+// and the atomic kernel, one persistent launch per thread count.
 static sim_status step_resident(voxsim_ctx* ctx, int n)
 {
     cudaStream_t s = ctx->stream;
+    if (!ctx->rows_robots.empty()) {
+        ResidentArgs a{};
+        a.pv = ctx->view();
+        a.corner_order = ctx->d_mass_corner.p;
+        a.cflags = ctx->d_cflags.p;
+        a.prm = ctx->d_prm.p;
+        a.x = ctx->d_x.p;
+        a.v = ctx->d_v.p;
+        a.sc = ctx->d_sc.p;
+        a.nsteps = n;
+        a.c = ctx->stepconst();
+        a.order = ctx->d_rows.p;
+        a.n_robots = (int)ctx->rows_robots.size();
+        a.queue = ctx->d_queue.p + 2 + ctx->atomic_groups.size();
+        a.max_mass = ctx->rows_max_corner;
+        VX_CK(cudaMemsetAsync(a.queue, 0, sizeof(int), s));
+        VX_LAUNCH(ctx, launch_step_rows(a, ctx->rows_nd, ctx->rows_max_mass, (size_t)ctx->smem_optin / 2 + 4096,
+                                        std::min(a.n_robots, ctx->num_sms), s));
+    }
     for (size_t gi = 0; gi < ctx->atomic_groups.size(); ++gi) {
         const voxsim_ctx::AtomicGroup& g = ctx->atomic_groups[gi];
         ResidentArgs a{};

@@ -168,12 +168,16 @@ struct ResidentArgs {
     int tm_rec;              // springs per thread held in tensor memory (0: none, nothing allocated)
     int tm_cols;             // tensor-memory columns per warp (of the block's 512)
     int accumulate;          // SIM_ACC_ATOMIC or SIM_ACC_GATHER
-    // gather path
-    const int* inc_off;      // [moff-based] per-mass incidence start (length M+1 per robot)
-    const int* inc_list;     // [soff*2-based] spring index * 2 + side
+    // step_rows.cu: the masses' corners (ascending), the parameter planes
+    const int* corner_order;
+    const float* prm;
 };
 cudaError_t launch_step_resident(const ResidentArgs& a, int grid, int threads, size_t smem,
                                  cudaStream_t s);
+
+// Robots with force rows in shared memory, undamped (step_rows.cu).
+int rows_per_corner(int corners, size_t budget);
+cudaError_t launch_step_rows(const ResidentArgs& a, int nd, int max_masses, size_t min_smem, int grid, cudaStream_t s);
 
 // Lattice-gather path (deterministic): work items of robots of one size class.
 struct LatticeArgs {
