@@ -91,6 +91,85 @@ struct DevBuf {
     ~DevBuf() { release(); }
 };
 
+// A stretch of another buffer.
+template <class T>
+struct DevRef {
+    T* p = nullptr;
+};
+
+// Pinned host memory through which small arrays travel: a copy from or to it is asynchronous and
+// costs one call, where each copy of ordinary memory waits for the stream (reads) or is staged by the
+// driver (writes).  begin() waits for the copies still using it, take() hands out 16-byte-aligned
+// pieces, end() marks the stream position after which it is free again.
+struct Staging {
+    unsigned char* p = nullptr;
+    size_t cap = 0, used = 0;
+    cudaEvent_t ev = nullptr;
+    bool pending = false;
+    static size_t padded(size_t bytes) { return (bytes + 15) / 16 * 16; }
+    cudaError_t begin(size_t want)
+    {
+        if (!ev) {
+            cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+            if (e != cudaSuccess) { ev = nullptr; return e; }
+        }
+        if (pending) {
+            cudaError_t e = cudaEventSynchronize(ev);
+            if (e != cudaSuccess) return e;
+            pending = false;
+        }
+        used = 0;
+        if (want > cap) {
+            if (p) cudaFreeHost(p);
+            p = nullptr;
+            cap = 0;
+            const size_t n = std::max<size_t>(want + want / 2, 1 << 16);
+            cudaError_t e = cudaMallocHost((void**)&p, n);
+            if (e != cudaSuccess) { p = nullptr; return e; }
+            cap = n;
+        }
+        return cudaSuccess;
+    }
+    unsigned char* take(size_t bytes)
+    {
+        unsigned char* q = p + used;
+        used += padded(bytes);
+        return q;
+    }
+    cudaError_t end(cudaStream_t s)
+    {
+        cudaError_t e = cudaEventRecord(ev, s);
+        pending = e == cudaSuccess;
+        return e;
+    }
+    void release()
+    {
+        if (pending) cudaEventSynchronize(ev);
+        if (ev) cudaEventDestroy(ev);
+        if (p) cudaFreeHost(p);
+        p = nullptr;
+        ev = nullptr;
+        cap = 0;
+        pending = false;
+    }
+};
+
+// Index of the first material id out of range, or -1; eight bytes at a time (a byte of at least 5
+// sets its top bit in the sum or has it set already).
+int64_t first_bad_material(const uint8_t* m, int64_t n)
+{
+    static_assert(kNumMat == 5, "the constant below is 0x80 - 5 per byte");
+    int64_t i = 0;
+    for (; i + 8 <= n; i += 8) {
+        uint64_t w;
+        std::memcpy(&w, m + i, 8);
+        if ((((w & 0x7f7f7f7f7f7f7f7full) + 0x7b7b7b7b7b7b7b7bull) | w) & 0x8080808080808080ull) break;
+    }
+    for (; i < n; ++i)
+        if (m[i] >= kNumMat) return i;
+    return -1;
+}
+
 struct DeviceGuard {
     int prev = -1;
     bool ok = true;
@@ -158,7 +237,6 @@ struct voxsim_ctx {
     int n_pitems = 0;
     bool pitems_cover_corner = false;   // the per-corner robots are in the packed plan too
     size_t pitem_smem = 0;
-    DevBuf<int4> d_pitems, d_pgroups;
     // imposed contact modes (sim_impose_contact_modes): per robot the offset of its table in
     // imp_table (-1: none), tables of imp_n steps x the robot's corners; device copies
     bool imp_active = false;
@@ -189,17 +267,14 @@ struct voxsim_ctx {
     // robots on the per-mass kernel of 1024-thread blocks (step_rows.cu): one persistent launch
     std::vector<int> rows_robots;
     int rows_max_corner = 0, rows_max_mass = 0, rows_nd = 0;
-    DevBuf<int> d_rows;
     // cluster lattice groups (one launch each): robots cut into q slabs
     struct ClusterGroup { int q; int first; int count; };
     std::vector<ClusterGroup> cluster_groups;
     int n_cluster = 0;
-    DevBuf<int> d_cluster;
     int n_stream = 0, max_stream_corner = 0;
     bool stream_cube40 = false;  // every streamed robot is 40 x 40 x 40
     bool corner_grid8 = false;   // every per-corner lattice item is one robot of at most 8 voxels per axis (768 threads)
     std::vector<int> stream_robots;
-    DevBuf<int> d_stream;
     // CUDA graph of the streamed N-step loop, cached by step count (captured on a private
     // non-blocking stream, replayed on the context's stream)
     cudaStream_t capture_stream = nullptr;
@@ -224,11 +299,22 @@ struct voxsim_ctx {
         stream_graph_every = 0;
     }
     // device buffers
-    DevBuf<int> d_dims;
-    DevBuf<int64_t> d_voff, d_moff, d_soff, d_tmp_off;
-    DevBuf<int> d_nm, d_ns, d_queue, d_status, d_item_robots, d_big, d_grad_rows;
+    Staging staging;
+    // the layout arrays, one buffer: voxel, corner and spring offsets, dims
+    DevBuf<int64_t> d_layout;
+    DevRef<int> d_dims;
+    DevRef<int64_t> d_voff, d_moff, d_soff;
+    DevBuf<int64_t> d_tmp_off;
+    // masses and springs per robot and the status words, one buffer
+    DevBuf<int> d_counts;
+    DevRef<int> d_nm, d_ns, d_status;
+    DevBuf<int> d_queue, d_grad_rows;
+    // the execution plan's lists, one buffer (build_work_items)
+    DevBuf<int4> d_plan;
+    DevRef<int> d_item_robots, d_big, d_stream, d_rows, d_cluster;
+    DevRef<int4> d_items, d_pitems, d_pgroups;
+    std::vector<int4> pitems, pgroups;
     DevBuf<int> d_progress;      // per lattice item: segments done (segmented queue)
-    DevBuf<int4> d_items;
     DevBuf<uint32_t> d_cflags;
     DevBuf<float> d_prm;
     DevBuf<uint8_t> d_in_u8, d_mat_raw, d_mat;
@@ -244,7 +330,6 @@ struct voxsim_ctx {
     DevBuf<int> d_topo_robots, d_zmin;
     DevBuf<unsigned long long> d_best;
     DevBuf<int2> d_chunk;
-    std::vector<int> topo_robots;   // (host copy of d_topo_robots: small robots, then large ones)
     DevBuf<int2> d_sab;
     DevBuf<float4> d_sp, d_spack, d_x0, d_x, d_v, d_x_alt, d_v_alt;
     DevBuf<float> d_plain_f;       // force accumulators of the plain path (3 per corner)
@@ -442,6 +527,7 @@ sim_status sim_destroy(voxsim_ctx* ctx)
     }
     for (cudaEvent_t e : ctx->ev_bwd)
         if (e) cudaEventDestroy(e);
+    ctx->staging.release();
     delete ctx;   // device buffers are released by their destructors
     return SIM_OK;
 }
@@ -495,8 +581,8 @@ sim_status sim_set_population(voxsim_ctx* ctx, int32_t P, const int32_t* dims, i
                            : mode == SIM_MODE_PARAMS  ? ((const sim_voxel_params*)genomes)->mat
                                                       : ((const sim_param_rows*)genomes)->mat;
         if (V > 0 && !m) return fail(SIM_EINVAL, "null materials");
-        for (int64_t i = 0; i < V; ++i)
-            if (m[i] >= kNumMat) return fail(SIM_EINVAL, "material id %d at voxel %lld", (int)m[i], (long long)i);
+        const int64_t i = first_bad_material(m, V);
+        if (i >= 0) return fail(SIM_EINVAL, "material id %d at voxel %lld", (int)m[i], (long long)i);
     }
     if (mode == SIM_MODE_PARAMS) {
         const sim_voxel_params* vp = (const sim_voxel_params*)genomes;
@@ -504,11 +590,18 @@ sim_status sim_set_population(voxsim_ctx* ctx, int32_t P, const int32_t* dims, i
             return fail(SIM_EINVAL, "null per-voxel parameter array");
     }
     // buffers
-    VX_CK(ctx->d_dims.ensure(3 * (size_t)P));
-    VX_CK(ctx->d_voff.ensure(P + 1)); VX_CK(ctx->d_moff.ensure(P + 1)); VX_CK(ctx->d_soff.ensure(P + 1));
+    const size_t n_off = 3 * ((size_t)P + 1), layout_bytes = sizeof(int64_t) * n_off + sizeof(int) * 3 * P;
+    VX_CK(ctx->d_layout.ensure(n_off + (3 * (size_t)P + 1) / 2));
+    ctx->d_voff.p = ctx->d_layout.p;
+    ctx->d_moff.p = ctx->d_voff.p + P + 1;
+    ctx->d_soff.p = ctx->d_moff.p + P + 1;
+    ctx->d_dims.p = reinterpret_cast<int*>(ctx->d_layout.p + n_off);
     VX_CK(ctx->d_tmp_off.ensure(P + 1));
-    VX_CK(ctx->d_nm.ensure(P)); VX_CK(ctx->d_ns.ensure(P));
-    VX_CK(ctx->d_queue.ensure(3)); VX_CK(ctx->d_status.ensure(4));
+    VX_CK(ctx->d_counts.ensure(2 * (size_t)P + 4));
+    ctx->d_nm.p = ctx->d_counts.p;
+    ctx->d_ns.p = ctx->d_nm.p + P;
+    ctx->d_status.p = ctx->d_ns.p + P;
+    VX_CK(ctx->d_queue.ensure(3));
     VX_CK(ctx->d_mat_raw.ensure(V)); VX_CK(ctx->d_mat.ensure(V));
     VX_CK(ctx->d_w.ensure(V)); VX_CK(ctx->d_kappa.ensure(V)); VX_CK(ctx->d_phi.ensure(V));
     VX_CK(ctx->d_vox_q.ensure(V)); VX_CK(ctx->d_vox_s.ensure(V));
@@ -529,10 +622,17 @@ sim_status sim_set_population(voxsim_ctx* ctx, int32_t P, const int32_t* dims, i
     ctx->max_corner = max_corner; ctx->max_spring_cap = max_sc;
     ctx->have_pop = false;
     if (P > 0) {
-        VX_CK(cudaMemcpyAsync(ctx->d_dims.p, d.data(), sizeof(int) * 3 * P, cudaMemcpyHostToDevice, s));
-        VX_CK(cudaMemcpyAsync(ctx->d_voff.p, voff.data(), sizeof(int64_t) * (P + 1), cudaMemcpyHostToDevice, s));
-        VX_CK(cudaMemcpyAsync(ctx->d_moff.p, moff.data(), sizeof(int64_t) * (P + 1), cudaMemcpyHostToDevice, s));
-        VX_CK(cudaMemcpyAsync(ctx->d_soff.p, soff.data(), sizeof(int64_t) * (P + 1), cudaMemcpyHostToDevice, s));
+        // room for this copy, the topology's robot list and the counts that come back
+        VX_CK(ctx->staging.begin(Staging::padded(layout_bytes) + Staging::padded(sizeof(int) * P) +
+                                 Staging::padded(sizeof(int) * (2 * (size_t)P + 4))));
+        unsigned char* h = ctx->staging.take(layout_bytes);
+        const size_t off_bytes = sizeof(int64_t) * (P + 1);
+        std::memcpy(h, voff.data(), off_bytes);
+        std::memcpy(h + off_bytes, moff.data(), off_bytes);
+        std::memcpy(h + 2 * off_bytes, soff.data(), off_bytes);
+        std::memcpy(h + 3 * off_bytes, d.data(), sizeof(int) * 3 * P);
+        VX_CK(cudaMemcpyAsync(ctx->d_layout.p, h, layout_bytes, cudaMemcpyHostToDevice, s));
+        VX_CK(ctx->staging.end(s));
     }
     VX_CK(cudaMemsetAsync(ctx->d_status.p, 0, 4 * sizeof(int), s));
     ctx->host_genome_floats = 0;
@@ -618,13 +718,15 @@ sim_status sim_set_population(voxsim_ctx* ctx, int32_t P, const int32_t* dims, i
         // topology
         if (sim_status st = run_topology(ctx, packed)) return st;
         // the mass counts order the work queue (longest first); the plan is built on the host
-        ctx->mass_count.assign(P, 0);
-        ctx->spring_count.assign(P, 0);
-        VX_CK(cudaMemcpyAsync(ctx->mass_count.data(), ctx->d_nm.p, sizeof(int) * P, cudaMemcpyDeviceToHost, s));
-        VX_CK(cudaMemcpyAsync(ctx->spring_count.data(), ctx->d_ns.p, sizeof(int) * P, cudaMemcpyDeviceToHost, s));
-        int32_t words[4] = {0, 0, 0, 0};
-        VX_CK(cudaMemcpyAsync(words, ctx->d_status.p, sizeof(words), cudaMemcpyDeviceToHost, s));
+        const size_t count_bytes = sizeof(int) * (2 * (size_t)P + 4);
+        int* h = reinterpret_cast<int*>(ctx->staging.take(count_bytes));
+        VX_CK(cudaMemcpyAsync(h, ctx->d_counts.p, count_bytes, cudaMemcpyDeviceToHost, s));
         VX_CK(cudaStreamSynchronize(s));
+        ctx->staging.pending = false;
+        ctx->mass_count.assign(h, h + P);
+        ctx->spring_count.assign(h + P, h + 2 * P);
+        int32_t words[4];
+        std::memcpy(words, h + 2 * P, sizeof(words));
         if (sim_status st = status_from_words(words)) return st;
         if (sim_status st = build_work_items(ctx)) return st;
     }
@@ -676,14 +778,14 @@ static sim_status run_topology(voxsim_ctx* ctx, bool packed)
     a.rest2 = (float)(ctx->p.edge * 1.4142135623730951);
     a.rest3 = (float)(ctx->p.edge * 1.7320508075688772);
     if (!large.empty()) {
-        // (the host copy lives in the context: the upload may still read it after this call)
-        ctx->topo_robots = small;
-        ctx->topo_robots.insert(ctx->topo_robots.end(), large.begin(), large.end());
         VX_CK(ctx->d_topo_robots.ensure(P));
         VX_CK(ctx->d_label.ensure(ctx->V_tot)); VX_CK(ctx->d_count.ensure(ctx->V_tot));
         VX_CK(ctx->d_best.ensure(P)); VX_CK(ctx->d_zmin.ensure(P));
         VX_CK(ctx->d_chunk.ensure(topology_chunks(cor[1]) * std::min<size_t>(large.size(), 32768)));
-        VX_CK(cudaMemcpyAsync(ctx->d_topo_robots.p, ctx->topo_robots.data(), sizeof(int) * P, cudaMemcpyHostToDevice, s));
+        int* h = reinterpret_cast<int*>(ctx->staging.take(sizeof(int) * P));   // (begun by the caller)
+        std::copy(large.begin(), large.end(), std::copy(small.begin(), small.end(), h));
+        VX_CK(cudaMemcpyAsync(ctx->d_topo_robots.p, h, sizeof(int) * P, cudaMemcpyHostToDevice, s));
+        VX_CK(ctx->staging.end(s));
         a.label = ctx->d_label.p;
         a.count = ctx->d_count.p;
         a.best = ctx->d_best.p;
@@ -969,35 +1071,39 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
                              ctx->dims[3 * r + 2] == 40;
     cudaStream_t s = ctx->stream;
     VX_CK(ctx->d_queue.ensure(3 + ctx->atomic_groups.size()));
-    VX_CK(ctx->d_rows.ensure(rows.size()));
-    if (!rows.empty())
-        VX_CK(cudaMemcpyAsync(ctx->d_rows.p, ctx->rows_robots.data(), sizeof(int) * rows.size(), cudaMemcpyHostToDevice, s));
+    VX_CK(ctx->d_progress.ensure(std::max(items.size(), ctx->pitems.size())));
     if (!streamed.empty()) {
-        VX_CK(ctx->d_stream.ensure(streamed.size()));
-        VX_CK(cudaMemcpyAsync(ctx->d_stream.p, streamed.data(), sizeof(int) * streamed.size(),
-                              cudaMemcpyHostToDevice, s));
         // both state buffers start equal (corners without a mass are never rewritten)
         VX_CK(ctx->d_x_alt.ensure(ctx->M_cap));
         VX_CK(ctx->d_v_alt.ensure(ctx->M_cap));
         VX_CK(cudaMemcpyAsync(ctx->d_x_alt.p, ctx->d_x.p, sizeof(float4) * ctx->M_cap, cudaMemcpyDeviceToDevice, s));
         VX_CK(cudaMemcpyAsync(ctx->d_v_alt.p, ctx->d_v.p, sizeof(float4) * ctx->M_cap, cudaMemcpyDeviceToDevice, s));
     }
-    VX_CK(ctx->d_items.ensure(items.size()));
-    VX_CK(ctx->d_progress.ensure(items.size()));
-    VX_CK(ctx->d_item_robots.ensure(robots.size()));
-    VX_CK(ctx->d_big.ensure(big.size()));
-    if (!items.empty()) {
-        VX_CK(cudaMemcpyAsync(ctx->d_items.p, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice, s));
-        VX_CK(cudaMemcpyAsync(ctx->d_item_robots.p, robots.data(), sizeof(int) * robots.size(), cudaMemcpyHostToDevice, s));
+    // all lists of the plan in one copy
+    size_t total = 0;
+    for (size_t bytes : {sizeof(int4) * items.size(), sizeof(int4) * ctx->pitems.size(), sizeof(int4) * ctx->pgroups.size(),
+                         sizeof(int) * robots.size(), sizeof(int) * big.size(), sizeof(int) * ctx->rows_robots.size(),
+                         sizeof(int) * cl_robots.size(), sizeof(int) * streamed.size()})
+        total += Staging::padded(bytes);
+    VX_CK(ctx->d_plan.ensure(total / sizeof(int4)));
+    if (total > 0) {
+        VX_CK(ctx->staging.begin(total));
+        auto put = [&](const auto& list, auto& ref) {
+            ref.p = reinterpret_cast<decltype(ref.p)>(reinterpret_cast<unsigned char*>(ctx->d_plan.p) + ctx->staging.used);
+            unsigned char* h = ctx->staging.take(sizeof(list[0]) * list.size());
+            if (!list.empty()) std::memcpy(h, list.data(), sizeof(list[0]) * list.size());
+        };
+        put(items, ctx->d_items);
+        put(ctx->pitems, ctx->d_pitems);
+        put(ctx->pgroups, ctx->d_pgroups);
+        put(robots, ctx->d_item_robots);
+        put(big, ctx->d_big);
+        put(ctx->rows_robots, ctx->d_rows);
+        put(cl_robots, ctx->d_cluster);
+        put(streamed, ctx->d_stream);
+        VX_CK(cudaMemcpyAsync(ctx->d_plan.p, ctx->staging.p, total, cudaMemcpyHostToDevice, s));
+        VX_CK(ctx->staging.end(s));
     }
-    if (!big.empty())
-        VX_CK(cudaMemcpyAsync(ctx->d_big.p, big.data(), sizeof(int) * big.size(), cudaMemcpyHostToDevice, s));
-    VX_CK(ctx->d_cluster.ensure(cl_robots.size()));
-    if (!cl_robots.empty())
-        VX_CK(cudaMemcpyAsync(ctx->d_cluster.p, cl_robots.data(), sizeof(int) * cl_robots.size(),
-                              cudaMemcpyHostToDevice, s));
-    // the host vectors are copied from pageable memory: wait so they may go out of scope
-    VX_CK(cudaStreamSynchronize(s));
     ctx->drop_graph();
     return SIM_OK;
 }
@@ -1014,6 +1120,8 @@ static sim_status build_packed_items(voxsim_ctx* ctx, const std::vector<std::vec
     ctx->n_pitems = 0;
     ctx->pitems_cover_corner = false;
     ctx->pitem_smem = 0;
+    ctx->pitems.clear();
+    ctx->pgroups.clear();
     const bool masses_known = (int)ctx->mass_count.size() == ctx->P;
     // the per-corner robots join the packed plan only when asked for: measured slower than the
     // one-robot-per-slot kernel on the workloads tried (its address arithmetic adds 22 %
@@ -1073,16 +1181,34 @@ static sim_status build_packed_items(voxsim_ctx* ctx, const std::vector<std::vec
     };
     struct Bin { int threads; size_t smem; std::vector<int> members; };
     std::vector<Bin> bins;
+    // first fit: a tree over the bins with the most threads free below each node leads to the next
+    // bin with room for T threads (0 once a bin holds 15 groups); bins past the last are all free
+    size_t leaves = 1;
+    while (leaves < gs.size()) leaves *= 2;
+    std::vector<int> room(2 * leaves, cap);
+    auto next_bin = [&](size_t from, int T) {            // the first bin >= from with room (one exists)
+        size_t i = leaves + from;
+        while (room[i] < T) {
+            while (i & 1) i /= 2;                        // up while a right child, then to the right
+            ++i;
+            if (room[i] < T) continue;
+            while (i < leaves) i = room[2 * i] >= T ? 2 * i : 2 * i + 1;
+        }
+        return i - leaves;
+    };
     for (int i = 0; i < (int)gs.size(); ++i) {
         const size_t b = need(gs[i]);
         if (b > budget) return fail(SIM_EINVAL, "robot %d does not fit a lattice block", gs[i].r);
-        Bin* home = nullptr;
-        for (Bin& bin : bins)
-            if (bin.threads + gs[i].T <= cap && bin.smem + b <= budget && bin.members.size() < 15) { home = &bin; break; }
-        if (!home) { bins.push_back({0, 0, {}}); home = &bins.back(); }
-        home->threads += gs[i].T;
-        home->smem += b;
-        home->members.push_back(i);
+        size_t at = next_bin(0, gs[i].T);
+        while (at < bins.size() && bins[at].smem + b > budget) at = next_bin(at + 1, gs[i].T);
+        if (at >= bins.size()) { at = bins.size(); bins.push_back({0, 0, {}}); }
+        Bin& home = bins[at];
+        home.threads += gs[i].T;
+        home.smem += b;
+        home.members.push_back(i);
+        size_t node = leaves + at;
+        room[node] = home.members.size() < 15 ? cap - home.threads : 0;
+        for (node /= 2; node >= 1; node /= 2) room[node] = std::max(room[2 * node], room[2 * node + 1]);
     }
     std::vector<int4> items, groups;
     for (const Bin& bin : bins) {
@@ -1096,13 +1222,8 @@ static sim_status build_packed_items(voxsim_ctx* ctx, const std::vector<std::vec
         }
         ctx->pitem_smem = std::max(ctx->pitem_smem, bin.smem);
     }
-    VX_CK(ctx->d_pitems.ensure(items.size()));
-    VX_CK(ctx->d_progress.ensure(items.size()));
-    VX_CK(ctx->d_pgroups.ensure(groups.size()));
-    VX_CK(cudaMemcpyAsync(ctx->d_pitems.p, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice, ctx->stream));
-    VX_CK(cudaMemcpyAsync(ctx->d_pgroups.p, groups.data(), sizeof(int4) * groups.size(), cudaMemcpyHostToDevice, ctx->stream));
-    // the host vectors go out of scope: the copies must have read them
-    VX_CK(cudaStreamSynchronize(ctx->stream));
+    ctx->pitems = items;
+    ctx->pgroups = groups;
     ctx->n_pitems = (int)items.size();
     return SIM_OK;
 }
@@ -1468,10 +1589,15 @@ sim_status sim_fitness(voxsim_ctx* ctx, double* out, int32_t mem)
                                   (float)ctx->p.dead_bound, fitness_chunks(ctx->max_corner), ctx->d_fit_part.p,
                                   ctx->d_fit_arrived.p, dst, s));
     if (mem == SIM_MEM_HOST) {
-        // the status words ride along: a segmented lattice step that gave up waiting shows here
-        int32_t words[4];
-        VX_CK(cudaMemcpyAsync(words, ctx->d_status.p, sizeof(words), cudaMemcpyDeviceToHost, s));
-        if (sim_status st = copy_out(out, ctx->d_fit.p, sizeof(double) * ctx->P, mem, s)) return st;
+        // the status words ride along: a step that gave up waiting shows here
+        const size_t fit_bytes = sizeof(double) * ctx->P;
+        VX_CK(ctx->staging.begin(Staging::padded(fit_bytes) + 4 * sizeof(int32_t)));
+        unsigned char* hf = ctx->staging.take(fit_bytes);
+        int32_t* words = reinterpret_cast<int32_t*>(ctx->staging.take(4 * sizeof(int32_t)));
+        VX_CK(cudaMemcpyAsync(words, ctx->d_status.p, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+        if (ctx->P > 0) VX_CK(cudaMemcpyAsync(hf, ctx->d_fit.p, fit_bytes, cudaMemcpyDeviceToHost, s));
+        VX_CK(cudaStreamSynchronize(s));
+        if (ctx->P > 0) std::memcpy(out, hf, fit_bytes);
         const int32_t step_words[4] = {0, 0, words[2], 0};   // the population's own were reported
         return status_from_words(step_words);
     }
@@ -1553,12 +1679,15 @@ sim_status evo_gradient_step(voxsim_ctx* ctx, float* genomes, int32_t P, int32_t
             if (rows[i] < 0 || rows[i] >= P) return fail(SIM_EINVAL, "row %d out of range", rows[i]);
             list.push_back(rows[i]);
         }
-    } else {
-        for (int r = 0; r < P; ++r) list.push_back(r);
+        if (list.empty()) return SIM_OK;
     }
-    if (list.empty()) return SIM_OK;
     DeviceGuard g(ctx->device);
     cudaStream_t s = ctx->stream;
+    if (!rows) {                                         // every row: no list
+        VX_LAUNCH(ctx, launch_grad_step(genomes, G, V, ctx->d_voff.p, g_w, g_kappa, g_phi, nullptr, P, eta_w, eta_kappa,
+                                        eta_phi, lo, hi, s));
+        return SIM_OK;
+    }
     VX_CK(ctx->d_grad_rows.ensure(list.size()));
     VX_CK(cudaMemcpyAsync(ctx->d_grad_rows.p, list.data(), sizeof(int) * list.size(), cudaMemcpyHostToDevice, s));
     VX_LAUNCH(ctx, launch_grad_step(genomes, G, V, ctx->d_voff.p, g_w, g_kappa, g_phi, ctx->d_grad_rows.p,
@@ -2102,10 +2231,10 @@ sim_status sim_get_counts(voxsim_ctx* ctx, int32_t* n_masses, int32_t* n_springs
     if (sim_status st = check_ctx(ctx)) return st;
     if (!ctx->have_pop) return fail(SIM_ESTATE, "no population set");
     DeviceGuard g(ctx->device);
-    cudaStream_t s = ctx->stream;
-    if (n_masses && ctx->P) VX_CK(cudaMemcpyAsync(n_masses, ctx->d_nm.p, 4 * ctx->P, cudaMemcpyDeviceToHost, s));
-    if (n_springs && ctx->P) VX_CK(cudaMemcpyAsync(n_springs, ctx->d_ns.p, 4 * ctx->P, cudaMemcpyDeviceToHost, s));
-    VX_CK(cudaStreamSynchronize(s));
+    // (sim_set_population has read the counts back for its plan)
+    if (n_masses && ctx->P) std::memcpy(n_masses, ctx->mass_count.data(), sizeof(int) * ctx->P);
+    if (n_springs && ctx->P) std::memcpy(n_springs, ctx->spring_count.data(), sizeof(int) * ctx->P);
+    VX_CK(cudaStreamSynchronize(ctx->stream));
     return SIM_OK;
 }
 

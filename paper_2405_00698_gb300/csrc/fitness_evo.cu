@@ -435,7 +435,7 @@ cudaError_t launch_diversity(const float* genomes, int P, int G, const uint8_t* 
 
 // ----------------------------------------------------------------------------------------------
 // Lamarckian gradient step on genome rows [w | kappa | phi] (gradient-assisted co-design): for
-// listed row r and gene j, genome <- clamp(fmaf(eta_seg, d, genome), lo_j, hi_j) with d the
+// listed row r (every row when there is no list) and gene j, genome <- clamp(fmaf(eta_seg, d, genome), lo_j, hi_j) with d the
 // adjoint's gradient of voxel j mod V of robot r (robot r's voxels start at voff[r]) and eta_seg
 // the step of the gene's segment.
 // ----------------------------------------------------------------------------------------------
@@ -448,7 +448,7 @@ __global__ void k_grad_step(float* __restrict__ genomes, int G, int64_t V, const
                             float eta_kappa, float eta_phi, const float* __restrict__ lo,
                             const float* __restrict__ hi)
 {
-    const int r = rows[blockIdx.y];
+    const int r = rows ? rows[blockIdx.y] : blockIdx.y;
     float* row = genomes + (size_t)r * G;
     const int64_t base = voff[r];
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < G; j += gridDim.x * blockDim.x) {
