@@ -141,25 +141,30 @@ __global__ void __launch_bounds__(kRankThreads) k_rank(const double* __restrict_
     }
 }
 
+// The generator's finaliser; high 32 bits.
+constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ull;
+__device__ __forceinline__ uint32_t mix(uint64_t z)
+{
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return (uint32_t)((z ^ (z >> 31)) >> 32);
+}
+
 // Draw number `purpose` of gene j of a row whose counters start at `ctr0` (generation and child
 // packed above gene and purpose): z = seed + (ctr + 1) gamma with the row's part added up before.
 __device__ __forceinline__ uint32_t row_draw(uint64_t z0, uint32_t j, uint32_t purpose)
 {
-    constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ull;
-    uint64_t z = z0 + (uint64_t)j * (8ull * kGamma) + purpose * kGamma;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return (uint32_t)((z ^ (z >> 31)) >> 32);
+    return mix(z0 + (uint64_t)j * (8ull * kGamma) + purpose * kGamma);
 }
 
 // A block takes kChildGenes genes of a row.  Elite rows copy their genome; child rows pick parents,
 // crossover mask and mutation from the counter-based generator.  A gene mutates with probability
 // 0.1 or so, so nearly every warp holds a mutating lane: the warp queues its mutating genes in
 // shared memory and evaluates the Gaussian for 32 of them at a time instead of for each warp of 32
-// genes (1024 genomes of 20,998 genes: 152 -> 78 us; 107 MB through device memory, 16 us; the
-// generator's 64-bit products are what is left).
+// genes (1024 genomes of 20,998 genes: 152 -> 66 us, 78 with one gene per lane in flight; 107 MB
+// through device memory, 16 us; the generator's 64-bit products are what is left).
 constexpr int kChildThreads = 256;
-constexpr int kChildGenes = 8 * kChildThreads;
+constexpr int kChildGenes = 16 * kChildThreads;
 
 __device__ __forceinline__ float mutated(uint64_t z0, uint32_t j, float g, float sigma)
 {
@@ -191,7 +196,7 @@ k_children(const float* __restrict__ gin, float* __restrict__ gout, const int* _
         }
         return;
     }
-    const uint64_t z0 = seed + (((((gen << 16) | (uint64_t)c) << 26) << 3) + 1ull) * 0x9E3779B97F4A7C15ull;
+    const uint64_t z0 = seed + (((((gen << 16) | (uint64_t)c) << 26) << 3) + 1ull) * kGamma;
     const uint32_t ua = row_draw(z0, 0, kParentA);
     const uint32_t ub = row_draw(z0, 0, kParentB);
     const int pa = order[(int)(((uint64_t)ua * (uint64_t)E) >> 32)];
@@ -208,30 +213,40 @@ k_children(const float* __restrict__ gin, float* __restrict__ gout, const int* _
     uint32_t* qj = sh_j[warp];
     float* qg = sh_g[warp];
     int queued = 0;                                       // of the warp, below 32 between rounds
-    for (int jb = j0 + 32 * warp; jb < j1; jb += kChildThreads) {
-        const int j = jb + lane;
-        bool mut = false;
-        float g = 0.f;
-        if (j < j1) {
-            const uint32_t m = copy_a ? 1u : row_draw(z0, j, kMask) >> 31;
-            g = m ? A[j] : Bp[j];
-            mut = row_draw(z0, j, kMutate) < thresh;
-            if (!mut) gout[row + j] = g;
-            if (mask) mask[row + j] = (uint8_t)m;
+    constexpr int kU = 4;                                // genes per lane and round
+    uint64_t z = z0 + (uint64_t)(j0 + 32 * kU * warp + lane) * (8ull * kGamma);
+    for (int jb = j0 + 32 * kU * warp; jb < j1;
+         jb += kU * kChildThreads, z += (uint64_t)kU * kChildThreads * (8ull * kGamma)) {
+        bool mut[kU];
+        float g[kU];
+        uint32_t m[kU];
+#pragma unroll
+        for (int i = 0; i < kU; ++i) {
+            const int j = jb + 32 * i + lane;
+            const uint64_t zi = z + (uint64_t)(32 * i) * (8ull * kGamma);
+            m[i] = copy_a ? 1u : mix(zi + kMask * kGamma) >> 31;
+            mut[i] = j < j1 && mix(zi + kMutate * kGamma) < thresh;
+            g[i] = j < j1 ? (m[i] ? A[j] : Bp[j]) : 0.f;
         }
-        const unsigned w = __ballot_sync(0xffffffffu, mut);
-        if (mut) {
-            const int at = queued + __popc(w & ((1u << lane) - 1u));
-            qj[at] = (uint32_t)j;
-            qg[at] = g;
-        }
-        queued += __popc(w);
-        __syncwarp();
-        if (queued >= 32) {
-            queued -= 32;                                 // the last 32 of the queue
-            const uint32_t jm = qj[queued + lane];
-            gout[row + jm] = mutated(z0, jm, qg[queued + lane], sigma);
+#pragma unroll
+        for (int i = 0; i < kU; ++i) {
+            const int j = jb + 32 * i + lane;
+            if (j < j1 && !mut[i]) gout[row + j] = g[i];
+            if (mask && j < j1) mask[row + j] = (uint8_t)m[i];
+            const unsigned w = __ballot_sync(0xffffffffu, mut[i]);
+            if (mut[i]) {
+                const int at = queued + __popc(w & ((1u << lane) - 1u));
+                qj[at] = (uint32_t)j;
+                qg[at] = g[i];
+            }
+            queued += __popc(w);
             __syncwarp();
+            if (queued >= 32) {
+                queued -= 32;                             // the last 32 of the queue
+                const uint32_t jm = qj[queued + lane];
+                gout[row + jm] = mutated(z0, jm, qg[queued + lane], sigma);
+                __syncwarp();
+            }
         }
     }
     if (lane < queued) gout[row + qj[lane]] = mutated(z0, qj[lane], qg[lane], sigma);
