@@ -212,7 +212,7 @@ sim_status sim_set_population(voxsim_ctx* ctx, int32_t P, const int32_t* dims, i
  * the horizontal force but never more than that force (with Table II's mu_s < mu_k it would
  * otherwise reverse it).  When checkpointing is on
  * (sim_set_checkpointing), the call records the states the adjoint needs.  With more lattice
- * work items than SMs (and at least 512 steps) the resident lattice step runs every item's steps
+ * work items than SMs (and at least 64 steps) the resident lattice step runs every item's steps
  * as segments from one queue, each segment waiting (bounded, on the device) for its robots'
  * previous one; the results are the same bits as whole runs.  A wait that gives up is reported
  * by the next sim_fitness into host memory (SIM_ETIMEOUT).
@@ -398,8 +398,8 @@ sim_status sim_diversity(voxsim_ctx* ctx, const float* genomes, int32_t P, int32
  * class 0 = lattice (per corner), 1 = atomic resident, 2 = streamed, 3 = lattice
  * (direction-compacted), 4 = cluster of lattice blocks (robots cut into slabs of whole corner
  * layers, one block each), 5 = lattice in thread groups sized by mass count (robots of more than
- * 768 corners but at most 768 masses; larger ones of the class take the atomic kernel, or the
- * cluster when bit-reproducibility is required), and the atomic kernel's block size.
+ * 768 corners but at most 768 masses; larger ones of the class take the per-mass or the atomic kernel
+ * as without tuning, or the cluster when bit-reproducibility is required), and the atomic kernel's block size.
  * Synchronises the stream.  Errors: SIM_ESTATE without a population, SIM_EINVAL. */
 sim_status sim_autotune(voxsim_ctx* ctx, int32_t n_steps, int32_t* kind_out, int32_t* threads_out);
 

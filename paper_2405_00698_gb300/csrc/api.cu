@@ -1071,7 +1071,7 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
                              ctx->dims[3 * r + 2] == 40;
     cudaStream_t s = ctx->stream;
     VX_CK(ctx->d_queue.ensure(3 + ctx->atomic_groups.size()));
-    VX_CK(ctx->d_progress.ensure(std::max(items.size(), ctx->pitems.size())));
+    VX_CK(ctx->d_progress.ensure(std::max({items.size(), ctx->pitems.size(), ctx->rows_robots.size()})));
     if (!streamed.empty()) {
         // both state buffers start equal (corners without a mass are never rewritten)
         VX_CK(ctx->d_x_alt.ensure(ctx->M_cap));
@@ -1242,14 +1242,29 @@ static sim_status timing_pair(voxsim_ctx* ctx, cudaEvent_t ev[2])
     return SIM_OK;
 }
 
-// Segments per item of the per-corner lattice launch: with more items than SMs, each item's n
-// steps are split so that the queue holds about 64 units per SM (at least 256 steps each); the
-// last wave then waits for one segment of the slowest items instead of one whole run.
+// Segments per item of a persistent launch (lattice, packed lattice, force rows): with more items
+// than SMs, each item's n steps are split, so that the last wave waits for one segment of the
+// slowest items instead of one whole run.  Among the splits with segments of at least kMinSegSteps
+// steps and at most kSegUnits units per SM, the one with the fewest step times on the busiest SM:
+// waves of units x (a unit's steps + its setup).  More segments are not always better: 250 robots
+// 5x5x5, 500 steps, take 1.62 ms in one (2 waves), 1.34 ms in 3 (5/3 waves) and 1.39 ms in 7 (12/7);
+// 600 robots 7x7x7 (3.95 waves), 500 steps, 3.80 ms in one and 3.88 ms in 7.
+// Against a fixed 64 units per SM of at least 256 steps from 512 steps on: 200 robots 6x9x5,
+// 500 steps, 2.18 -> 1.37 ms, 1000 robots 4x4x4 2.36 -> 1.35 ms, 500 robots 9x9x9 on the force rows
+// 3.42 -> 2.90 ms, 1024 robots 7x8x7 13.81 -> 13.69 ms, 1024 robots 8x8x8 (2000 steps) 29.27 ms both.
+// A least segment of 24, 48 or 64 steps: within 1 %.
+constexpr int kMinSegSteps = 32, kSegUnits = 32, kSegSetupSteps = 2;
 static int lattice_segments(int items, int n, int sms)
 {
-    if (items <= sms || n < 512) return 1;
-    const int want = (64 * sms + items - 1) / items, cap = n / 256;
-    return std::max(1, std::min(want, cap));
+    if (items <= sms) return 1;
+    const int cap = std::min(n / kMinSegSteps, (kSegUnits * sms + items - 1) / items);
+    int best = 1;
+    int64_t best_cost = INT64_MAX;
+    for (int k = 1; k <= std::max(1, cap); ++k) {
+        const int64_t waves = ((int64_t)items * k + sms - 1) / sms, cost = waves * ((n + k - 1) / k + kSegSetupSteps);
+        if (cost < best_cost) { best_cost = cost; best = k; }
+    }
+    return best;
 }
 
 // record: the call is sim_step_n's with checkpointing on (checkpoints, and the whole-trajectory
@@ -1379,6 +1394,11 @@ static sim_status step_resident(voxsim_ctx* ctx, int n)
         a.n_robots = (int)ctx->rows_robots.size();
         a.queue = ctx->d_queue.p + 2 + ctx->atomic_groups.size();
         a.max_mass = ctx->rows_max_corner;
+        a.nseg = lattice_segments(a.n_robots, n, ctx->num_sms);
+        a.seg_steps = (n + a.nseg - 1) / a.nseg;
+        a.progress = ctx->d_progress.p;
+        a.status = ctx->d_status.p + 2;
+        VX_CK(cudaMemsetAsync(a.progress, 0, sizeof(int) * a.n_robots, s));
         VX_CK(cudaMemsetAsync(a.queue, 0, sizeof(int), s));
         VX_LAUNCH(ctx, launch_step_rows(a, ctx->rows_nd, ctx->rows_max_mass, (size_t)ctx->smem_optin / 2 + 4096,
                                         std::min(a.n_robots, ctx->num_sms), s));

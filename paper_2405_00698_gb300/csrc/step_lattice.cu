@@ -7,18 +7,21 @@
 // (k, alpha L0, beta L0) of its up-to-13 forward springs.  Per step:
 //   phase A: for each forward spring (c, c + off(d)) the owner computes the force f from its own
 //            u and the neighbour's u (shared memory), adds f to its own total and writes f to
-//            the force plane d of shared memory at index c;
-//   phase B: each thread subtracts the plane-d entries at c - off(d) of its backward springs, then
+//            row 13 c + d of the force rows in shared memory;
+//   phase B: each thread subtracts rows 13 (c - off(d)) + d of its backward springs, then
 //            applies gravity, ground contact with friction and the semi-implicit Euler update in
 //            registers and publishes its new u.
-// Two block barriers per step, no atomics, and a fixed summation order (own forward springs by
-// direction, then backward springs by direction): bit-reproducible.
-// Shared memory per robot slot: u and v (float4 per corner) + 13 float4 force planes.
+// Two waits per step (barriers of the robot's group, or of neighbouring warps, WarpFlow), no
+// atomics, and a fixed summation order (own forward springs by direction, then backward springs by
+// direction): bit-reproducible.
+// Shared memory per robot slot: u, v and 13 force rows per corner, a float4 each, or 12 bytes in the
+// instantiations with compile-time strides (shared_rows.cuh).
 // The state is the displacement from the rest lattice (rest height z0 in u.w), so a spring
 // vector is d0 + (u_b - u_a) with d0 the exact lattice offset and the extension is formed without
 // cancellation: l - L0 = (2 d0.du + du.du) / (l + L0).
 #include "common.cuh"
 #include "physics.cuh"
+#include "segments.cuh"
 #include "shared_rows.cuh"
 #include "warp_flow.cuh"
 
@@ -26,22 +29,6 @@ namespace vx {
 namespace {
 
 constexpr int kMaxLatticeThreads = 768;
-// Polls of a segment's wait on its item's previous segment (each with a 256 ns sleep) before it
-// gives up: a few seconds, far beyond any segment's duration.
-constexpr uint32_t kSegSpinLimit = 1u << 22;
-
-__device__ __forceinline__ int ld_acquire_gpu(const int* p)
-{
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ void st_release_gpu(int* p, int v)
-{
-    asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
 __device__ __forceinline__ void group_sync(int id, int nthreads)
 {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
@@ -57,7 +44,8 @@ __device__ __forceinline__ void group_sync(int id, int nthreads)
 // are compile-time constants and the addresses of the 13 directions immediate offsets; the rows
 // are the narrow ones, and the warps wait for their neighbours (WarpFlow) instead of for the
 // group: 1024 MLP robots 8x8x8, 2000 steps: 32.8 ms with the group's barriers and float4 rows in
-// 13 planes, 31.7 ms with narrow rows, 29.9 ms with the neighbour waits too.  With run-time strides
+// 13 planes, 31.7 ms with narrow rows, 29.3 ms with the neighbour waits too; 1024 robots 7x8x7, 1000
+// steps: 15.4 -> 13.8 ms.  With run-time strides
 // the neighbour waits measured within 1 % of the barriers (12 % slower on groups of four warps),
 // narrow rows slower.
 template <bool DAMPED, bool RECORD, bool IMPOSE, bool GRID8 = false>
@@ -149,7 +137,7 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice(LatticeA
                 // phase A: forward springs (c, c + offset(d)).  No branch per direction: an
                 // absent spring has zero parameters and takes the corner itself as its far end
                 // (du = 0, so ext = 0 and the force is an exact zero that leaves the sums' bits
-                // unchanged); its plane entry is never read.  6.5 % faster than skipping it, and
+                // unchanged); its force row is never read.  6.5 % faster than skipping it, and
                 // 2.6 % more with the far end's load predicated off (u from the register).
                 auto forward = [&](auto t) {
                     constexpr int d = decltype(t)::value;
@@ -546,16 +534,16 @@ __global__ void __launch_bounds__(kMaxLatticeThreads, 1) k_step_lattice_compact(
 // evolved 8x8x8 robot of ~400 masses leaves half of a 768-thread block idle.  Here a block's
 // 768 threads are shared by several robots, each group sized by its mass count (a multiple of
 // 32 threads), so a block runs as many masses as it has threads.  What makes that fit in shared
-// memory is indexing the force planes by the thread slot of the spring's far end (the reader)
-// instead of by corner: a robot needs 13 planes of T entries (T = its threads) and its
-// displacements by corner (C entries), not 13 planes of C entries.  The far end's slot rides in
-// an integer beside the z of its shared displacement, which the spring evaluation loads anyway.
+// memory is grouping the force rows by the thread slot of the spring's far end (the reader)
+// instead of by corner: a robot needs 13 rows per thread (T threads) and its displacements by
+// corner (C entries), not 13 rows per corner.  The far end's slot rides in
+// the .w lane of its shared displacement, which the spring evaluation loads anyway.
 // Per step:
 //   phase A: for each forward spring (c, c + off(d)) the owner computes the force f from its own
-//            displacement and the far end's, adds f to its own total, and writes f into plane d
-//            at the far end's slot (absent springs write a never-read row per lane);
-//   phase B: each thread subtracts the plane-d entries at its own slot for its backward springs
-//            (contiguous, conflict-free rows), then the mass update.
+//            displacement and the far end's, adds f to its own total, and writes f into row d
+//            of the far end's slot (absent springs write a never-read row per lane);
+//   phase B: each thread subtracts its own slot's rows of its backward springs (contiguous,
+//            conflict-free), then the mass update.
 // The sums run over the same values in the same order as the per-corner kernel (own forward
 // springs by direction, then backward springs by direction): identical bits, so the adjoint's
 // replay (which runs the per-corner kernel) reproduces a run of this one.

@@ -13,12 +13,15 @@
 // The spring parameters of a thread's first mass and of 6 of its second mass's 13 springs live in
 // tensor memory (64 of its cells per thread); the others come from the parameter planes (L2) every
 // step.
+// With more robots than SMs a call's steps run in segments, as in k_step_lattice_seg, the robot's state
+// read and published through L2.
 // What bounds it: issue and the shared-memory pipe.  Against the atomic kernel, 200 steps: 500 robots
-// 9x9x9 of 1000 masses 6.28 -> 3.42 ms, 300 robots 10x10x10 of 1300 masses 3.69 -> 2.73 ms, 150 robots
+// 9x9x9 of 1000 masses 6.28 -> 3.42 ms (2.90 in segments), 300 robots 10x10x10 of 1300 masses 3.69 -> 2.73 ms, 150 robots
 // 11x10x12 of 1700 masses (two passes) 2.62 -> 1.63 ms, 152 full 12x12x12 3.15 -> 2.41 ms.  The row
 // addresses are formed anew in every pass: hoisted out of the steps they spilled 300 to 400 bytes.
 #include "common.cuh"
 #include "physics.cuh"
+#include "segments.cuh"
 #include "shared_rows.cuh"
 #include "tmem.cuh"
 
@@ -93,7 +96,7 @@ __device__ __forceinline__ void move_mass(float4& u, float4& v, float fx, float 
 template <int ND, int PER>
 __global__ void __launch_bounds__(kRowsThreads, 1) k_step_rows(ResidentArgs a)
 {
-    __shared__ int sh_robot;
+    __shared__ int sh_robot, sh_item, sh_begin, sh_end, sh_seg;
     __shared__ uint32_t sh_tmem;
     const int tid = threadIdx.x, warp = tid >> 5;
     const StepConst c = a.c;
@@ -106,8 +109,21 @@ __global__ void __launch_bounds__(kRowsThreads, 1) k_step_rows(ResidentArgs a)
     const NarrowRows su(0, cap), fb(12 * cap, ND * cap);
     for (;;) {
         if (tid == 0) {
-            const int i = atomicAdd(a.queue, 1);
-            sh_robot = i < a.n_robots ? a.order[i] : -1;
+            // unit it: segment it / n_robots of a robot, waiting (bounded) for the robot's previous
+            // segment, as in k_step_lattice_seg
+            const int it = atomicAdd(a.queue, 1), seg = it / a.n_robots, i = it - seg * a.n_robots;
+            sh_robot = seg < a.nseg ? a.order[i] : -1;
+            sh_item = i;
+            sh_seg = seg;
+            sh_begin = seg * a.seg_steps;
+            sh_end = min(sh_begin + a.seg_steps, a.nsteps);
+            if (seg > 0 && seg < a.nseg) {
+                uint32_t k = 0;
+                while (ld_acquire_gpu(a.progress + i) < seg) {
+                    if (++k >= kSegSpinLimit) { atomicOr(a.status, 8); break; }
+                    __nanosleep(256);
+                }
+            }
         }
         __syncthreads();
         const int r = sh_robot;
@@ -125,8 +141,9 @@ __global__ void __launch_bounds__(kRowsThreads, 1) k_step_rows(ResidentArgs a)
             const bool in = m < M;
             cidx[j] = in ? a.corner_order[mo + m] : 0;
             fl[j] = in ? a.cflags[mo + cidx[j]] : 0u;
-            u[j] = in ? a.x[mo + cidx[j]] : make_float4(0.f, 0.f, 0.f, 0.f);
-            v[j] = in ? a.v[mo + cidx[j]] : make_float4(0.f, 0.f, 0.f, 0.f);
+            // (the previous segment's state, written by another SM: read through L2)
+            u[j] = in ? __ldcg(a.x + mo + cidx[j]) : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[j] = in ? __ldcg(a.v + mo + cidx[j]) : make_float4(0.f, 0.f, 0.f, 0.f);
             if (in) {
                 su.store(cidx[j], u[j].x, u[j].y, u[j].z);
             }
@@ -153,7 +170,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1) k_step_rows(ResidentArgs a)
         });
         tmem_wait_st();
         __syncthreads();
-        for (int n = 0; n < a.nsteps; ++n) {
+        for (int n = sh_begin; n < *(volatile int*)&sh_end; ++n) {
             const float2 sc = a.sc[n];
             float2 Fxy[PER];
             float Fz[PER];
@@ -232,7 +249,9 @@ __global__ void __launch_bounds__(kRowsThreads, 1) k_step_rows(ResidentArgs a)
                 a.x[mo + cidx[j]] = u[j];
                 a.v[mo + cidx[j]] = v[j];
             }
+        __threadfence();                              // visible before the segment is published
         __syncthreads();
+        if (tid == 0) st_release_gpu(a.progress + sh_item, sh_seg + 1);
     }
     tmem_fence_before();                              // every thread has waited for its own accesses
     __syncthreads();

@@ -15,7 +15,7 @@
 // The waits are bounded; one that gives up returns false.
 //
 // What it gives: 1024 MLP robots 8x8x8 (20 warps each), 2000 steps: 31.7 ms with the group's
-// barriers, 29.9 ms with these waits; the adjoint's sweep gains with it too.  (test_wait in place of
+// barriers, 29.3 ms with these waits; the adjoint's sweep gains with it too.  (test_wait in place of
 // try_wait: 31.5 ms.)  A group of few warps gains nothing, since nearly all of its warps wait for
 // one another anyway and a barrier is quicker than an mbarrier's round trip (1000 robots 4x4x4 of
 // four warps, 500 steps: 2.35 ms with barriers, 2.64 ms with these waits): the kernels with

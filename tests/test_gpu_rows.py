@@ -58,3 +58,12 @@ def test_queue_repeats_and_agrees_with_streamed():
     s = run(pop, (20,), path=vs.PATH_STREAMED)
     assert np.array_equal(a[2], s[2])
     assert np.abs(a[0] - s[0]).max() <= 1e-6
+
+
+def test_segments_repeat_the_whole_run():
+    """More robots than SMs: the steps of one call run in segments from 64 steps on; the state must be
+    that of calls too short to be cut, bit for bit."""
+    pop = population(23, copies=34)
+    a, b = run(pop, (165,)), run(pop, (60, 60, 45))
+    for p, q in zip(a, b):
+        assert np.array_equal(p, q)
