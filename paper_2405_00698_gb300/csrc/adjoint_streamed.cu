@@ -31,14 +31,16 @@ struct CornerRef {
 template <int NC = 0>
 __device__ __forceinline__ bool corner_ref(const StreamAdjArgs& a, CornerRef& q)
 {
-    q.r = a.robots[blockIdx.y];
-    const int nx = a.pv.dims[3 * q.r], ny = a.pv.dims[3 * q.r + 1], nz = a.pv.dims[3 * q.r + 2];
-    q.X = NC ? NC + 1 : nx + 1;
-    q.XY = NC ? (NC + 1) * (NC + 1) : (nx + 1) * (ny + 1);
-    q.C = NC ? (NC + 1) * (NC + 1) * (NC + 1) : q.XY * (nz + 1);
+    StreamRobot s;
+    if constexpr (NC == 0) s = stream_robot(a);
+    else s.r = a.robots[blockIdx.y];
+    q.r = s.r;
+    q.X = NC ? NC + 1 : s.X;
+    q.XY = NC ? (NC + 1) * (NC + 1) : s.XY;
+    q.C = NC ? (NC + 1) * (NC + 1) * (NC + 1) : s.C;
     q.cidx = blockIdx.x * blockDim.x + threadIdx.x;
     if (q.cidx >= q.C) return false;
-    q.mo = a.pv.moff[q.r];
+    q.mo = NC ? a.pv.moff[q.r] : s.mo;
     q.fl = a.cflags[q.mo + q.cidx];
     return (q.fl >> 31) != 0u;                  // corners without a mass take no part
 }

@@ -245,6 +245,15 @@ struct voxsim_ctx {
     std::vector<uint8_t> imp_table;
     DevBuf<uint8_t> d_imp_modes;
     DevBuf<int64_t> d_imp_off;
+    // the streamed robots' grids for a launch's arguments, where they are few
+    void stream_table(StreamRobot* t) const
+    {
+        for (int i = 0; i < n_stream && n_stream <= kStreamTable; ++i) {
+            const int r = stream_robots[i], X = dims[3 * r] + 1, XY = X * (dims[3 * r + 1] + 1);
+            t[i] = {r, X, XY, XY * (dims[3 * r + 2] + 1), (int64_t)moff[r]};
+        }
+    }
+
     void imposed_args(LatticeArgs& a, int64_t step0) const
     {
         if (!imp_active) return;
@@ -1485,7 +1494,9 @@ static sim_status enqueue_streamed(voxsim_ctx* ctx, int n, cudaStream_t s, bool 
     a.c = ctx->stepconst();
     a.robots = ctx->d_stream.p;
     a.n_robots = ctx->n_stream;
+    ctx->stream_table(a.tab);
     a.cube40 = ctx->stream_cube40 ? 1 : 0;
+    a.n_sms = ctx->num_sms;
     const int K = record ? ctx->ckpt_every : 0;
     const bool keep = record && ctx->keep_records;
     for (int i = 0; i < n; ++i) {
@@ -1903,6 +1914,7 @@ static sim_status backward_streamed(voxsim_ctx* ctx, const double* dL_df)
     b.robots = ctx->d_stream.p;
     b.cube40 = ctx->stream_cube40 ? 1 : 0;
     b.n_robots = ctx->n_stream;
+    ctx->stream_table(b.tab);
     b.g_k = ctx->d_gk.p;
     b.g_a = ctx->d_ga.p;
     b.g_b = ctx->d_gb.p;
@@ -1919,7 +1931,9 @@ static sim_status backward_streamed(voxsim_ctx* ctx, const double* dL_df)
     f.c = ctx->stepconst();
     f.robots = ctx->d_stream.p;
     f.n_robots = ctx->n_stream;
+    ctx->stream_table(f.tab);
     f.cube40 = ctx->stream_cube40 ? 1 : 0;
+    f.n_sms = ctx->num_sms;
     const int nseg = (N + K - 1) / K;
     for (int seg = nseg - 1; seg >= 0; --seg) {
         const int n0 = seg * K, n1 = std::min(N, n0 + K);
@@ -2021,7 +2035,9 @@ sim_status sim_get_contact_modes(voxsim_ctx* ctx, int32_t robot, uint8_t* out)
             f.c = ctx->stepconst();
             f.robots = ctx->d_stream.p;
             f.n_robots = ctx->n_stream;
+            ctx->stream_table(f.tab);
             f.cube40 = ctx->stream_cube40 ? 1 : 0;
+            f.n_sms = ctx->num_sms;
             float4* ru[2] = {ctx->d_rep_u0.p, ctx->d_rep_u1.p};
             float4* rv[2] = {ctx->d_rep_v0.p, ctx->d_rep_v1.p};
             for (int i = 0; i < n1 - n0; ++i) {

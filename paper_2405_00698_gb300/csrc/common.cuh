@@ -237,6 +237,13 @@ struct LatticeArgs {
 };
 
 // Streamed path (robots too large for one SM): one launch per step over all their corners.
+// A streamed robot's grid (X corners per row, XY per layer, C in all) and the offset of its corners.
+struct StreamRobot {
+    int r, X, XY, C;
+    int64_t mo;
+};
+constexpr int kStreamTable = 16;
+
 struct StreamArgs {
     PopView pv;
     const uint32_t* cflags;
@@ -249,7 +256,9 @@ struct StreamArgs {
     StepConst c;
     const int* robots;       // streamed robots (grid.y)
     int n_robots;
+    StreamRobot tab[kStreamTable];   // the same with their grids, for at most kStreamTable robots
     int cube40;              // every streamed robot is 40 x 40 x 40 (compile-time strides)
+    int n_sms;
     // checkpoint of the state at the start of this step (NULL: none), per corner
     float4* ckpt_u;
     float4* ckpt_v;
@@ -258,6 +267,25 @@ struct StreamArgs {
     float4* rec_u;
     float2* rec_f;
 };
+#ifdef __CUDACC__
+// The launch's blockIdx.y-th robot.  Few robots: from the launch's arguments, since a launch of about
+// one wave is bound by its chain of loads, of which the list and the grid are two links (5 robots
+// 37x22x29: 9.9 -> 9.6 us per step; 4 robots 28x28x28, 100 steps with their gradient: 4.40 -> 4.22 ms).
+// Not with compile-time strides: the 40^3 step's code, which fills its registers, came out 18 %
+// slower with it.
+template <class Args>
+__device__ __forceinline__ StreamRobot stream_robot(const Args& a)
+{
+    if (a.n_robots <= kStreamTable) return a.tab[blockIdx.y];
+    StreamRobot q;
+    q.r = a.robots[blockIdx.y];
+    q.X = a.pv.dims[3 * q.r] + 1;
+    q.XY = q.X * (a.pv.dims[3 * q.r + 1] + 1);
+    q.C = q.XY * (a.pv.dims[3 * q.r + 2] + 1);
+    q.mo = a.pv.moff[q.r];
+    return q;
+}
+#endif
 cudaError_t launch_step_streamed(const StreamArgs& a, int n, int max_corners, cudaStream_t s);
 
 // Streamed adjoint (robots too large for one SM): records, adjoints and the per-spring
@@ -283,6 +311,7 @@ struct StreamAdjArgs {
     StepConst c;
     const int* robots;       // streamed robots (grid.y)
     int n_robots;
+    StreamRobot tab[kStreamTable];   // the same with their grids, for at most kStreamTable robots
     int cube40;              // every streamed robot is 40 x 40 x 40 (compile-time strides)
     float* g_k;              // per voxel accumulators
     float* g_a;

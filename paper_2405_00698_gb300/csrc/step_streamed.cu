@@ -29,17 +29,24 @@ constexpr int kStreamMinBlocks = 8;
 // NC > 0: every robot of the launch is NC x NC x NC (the large-robot workload's 40^3 grid): the
 // strides and plane size are compile-time constants, so the 13 neighbour and 39 parameter
 // addresses are immediate offsets (12.7 % faster on 64 robots 40^3, same bits).
-template <int NC>
-__global__ void __launch_bounds__(kStreamThreads, kStreamMinBlocks)
+// UNDAMPED: no dashpots (otherwise the launch's constants tell).  Without their code the run-time
+// strides leave room for 9 blocks per SM (56 registers), which a launch of several waves
+// takes (20 steps: 100 robots 18x40x17 1.84 -> 1.70 ms, 48 of 17x30x40 1.49 -> 1.37 ms, 32 of 24^3
+// 0.74 -> 0.67 ms).
+// One that all runs at once keeps 8: 5 robots 37x22x29 (1025 blocks) 9.8 us per step, 10.1 with 9.
+// The 40^3 instantiation stays as it is: 217 us per step on 64 robots, 229 without the dashpots'
+// code, 227 / 233 / 249 with 7 blocks per SM and batches of 5 or 6 or 6 blocks and batches of 7.
+template <int NC, bool UNDAMPED, int MINB>
+__global__ void __launch_bounds__(kStreamThreads, MINB)
 k_step_streamed(StreamArgs a, int n)
 {
-    const int r = a.robots[blockIdx.y];
-    const int nx = a.pv.dims[3 * r], ny = a.pv.dims[3 * r + 1], nz = a.pv.dims[3 * r + 2];
-    const int X = NC ? NC + 1 : nx + 1, XY = NC ? (NC + 1) * (NC + 1) : (nx + 1) * (ny + 1),
-              C = NC ? (NC + 1) * (NC + 1) * (NC + 1) : XY * (nz + 1);
+    StreamRobot q;
+    if constexpr (NC == 0) q = stream_robot(a);
+    else q.r = a.robots[blockIdx.y];
+    const int X = NC ? NC + 1 : q.X, XY = NC ? (NC + 1) * (NC + 1) : q.XY, C = NC ? (NC + 1) * (NC + 1) * (NC + 1) : q.C;
     const int cidx = blockIdx.x * blockDim.x + threadIdx.x;
     if (cidx >= C) return;
-    const int64_t mo = a.pv.moff[r];
+    const int64_t mo = NC ? a.pv.moff[q.r] : q.mo;
     const uint32_t fl = a.cflags[mo + cidx];
     if (!(fl >> 31)) return;                    // no mass here: nothing moves
     const float4* __restrict__ uin = a.u_in + mo;
@@ -80,7 +87,7 @@ k_step_streamed(StreamArgs a, int n)
             constexpr int d = decltype(t)::value, i = d - d0;
             SpringEval e = spring_eval_dir<d>(__fsub_rn(ub[i].x, u.x), __fsub_rn(ub[i].y, u.y), __fsub_rn(ub[i].z, u.z),
                                               c.edge, lattice_rest<d>(c), lattice_rest_sq<d>(c), pk[i], pa[i], pb[i], sc.x, sc.y);
-            if (c.damped) {
+            if (!UNDAMPED && c.damped) {
                 const float4 vb = vin[((fl >> d) & 1u) ? cidx + lattice_offset<d>(X, XY) : cidx];
                 spring_dashpot(e, __fsub_rn(vb.x, v.x), __fsub_rn(vb.y, v.y), __fsub_rn(vb.z, v.z), pk[i], c);
             }
@@ -105,7 +112,7 @@ k_step_streamed(StreamArgs a, int n)
             constexpr int d = decltype(t)::value, i = d - d0;
             SpringEval e = spring_eval_dir<d>(__fsub_rn(u.x, ua[i].x), __fsub_rn(u.y, ua[i].y), __fsub_rn(u.z, ua[i].z),
                                               c.edge, lattice_rest<d>(c), lattice_rest_sq<d>(c), pk[i], pa[i], pb[i], sc.x, sc.y);
-            if (c.damped) {
+            if (!UNDAMPED && c.damped) {
                 const float4 va = vin[((fl >> (16 + d)) & 1u) ? cidx - lattice_offset<d>(X, XY) : cidx];
                 spring_dashpot(e, __fsub_rn(v.x, va.x), __fsub_rn(v.y, va.y), __fsub_rn(v.z, va.z), pk[i], c);
             }
@@ -128,8 +135,11 @@ cudaError_t launch_step_streamed(const StreamArgs& a, int n, int max_corners, cu
 {
     if (a.n_robots == 0) return cudaSuccess;
     dim3 grid((max_corners + kStreamThreads - 1) / kStreamThreads, a.n_robots);
-    if (a.cube40) k_step_streamed<40><<<grid, kStreamThreads, 0, s>>>(a, n);
-    else k_step_streamed<0><<<grid, kStreamThreads, 0, s>>>(a, n);
+    const bool one_wave = (int64_t)grid.x * grid.y <= (int64_t)a.n_sms * kStreamMinBlocks;
+    auto kernel = a.cube40 ? k_step_streamed<40, false, kStreamMinBlocks>
+                : a.c.damped ? k_step_streamed<0, false, kStreamMinBlocks>
+                : one_wave ? k_step_streamed<0, true, kStreamMinBlocks> : k_step_streamed<0, true, kStreamMinBlocks + 1>;
+    kernel<<<grid, kStreamThreads, 0, s>>>(a, n);
     return cudaGetLastError();
 }
 
