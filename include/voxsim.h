@@ -398,8 +398,8 @@ sim_status sim_diversity(voxsim_ctx* ctx, const float* genomes, int32_t P, int32
  * class 0 = lattice (per corner), 1 = atomic resident, 2 = streamed, 3 = lattice
  * (direction-compacted), 4 = cluster of lattice blocks (robots cut into slabs of whole corner
  * layers, one block each), 5 = lattice in thread groups sized by mass count (robots of more than
- * 768 corners but at most 768 masses; larger ones of the class take the per-mass or the atomic kernel
- * as without tuning, or the cluster when bit-reproducibility is required), and the atomic kernel's block size.
+ * 768 corners but at most 768 masses; larger ones of the class take the atomic kernel, or the
+ * cluster when bit-reproducibility is required), and the atomic kernel's block size.
  * Synchronises the stream.  Errors: SIM_ESTATE without a population, SIM_EINVAL. */
 sim_status sim_autotune(voxsim_ctx* ctx, int32_t n_steps, int32_t* kind_out, int32_t* threads_out);
 

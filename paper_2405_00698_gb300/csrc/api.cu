@@ -273,9 +273,6 @@ struct voxsim_ctx {
     // atomic-kernel groups (one persistent launch each): robots of one thread count
     struct AtomicGroup { int threads; int first; int count; int max_corner; int64_t max_spring_cap; };
     std::vector<AtomicGroup> atomic_groups;
-    // robots on the per-mass kernel of 1024-thread blocks (step_rows.cu): one persistent launch
-    std::vector<int> rows_robots;
-    int rows_max_corner = 0, rows_max_mass = 0, rows_nd = 0;
     // cluster lattice groups (one launch each): robots cut into q slabs
     struct ClusterGroup { int q; int first; int count; };
     std::vector<ClusterGroup> cluster_groups;
@@ -320,7 +317,7 @@ struct voxsim_ctx {
     DevBuf<int> d_queue, d_grad_rows;
     // the execution plan's lists, one buffer (build_work_items)
     DevBuf<int4> d_plan;
-    DevRef<int> d_item_robots, d_big, d_stream, d_rows, d_cluster;
+    DevRef<int> d_item_robots, d_big, d_stream, d_cluster;
     DevRef<int4> d_items, d_pitems, d_pgroups;
     std::vector<int4> pitems, pgroups;
     DevBuf<int> d_progress;      // per lattice item: segments done (segmented queue)
@@ -878,7 +875,6 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
     ctx->atomic_groups.clear();
     if (ctx->p.path == SIM_PATH_PLAIN) {       // every robot on the baseline kernels
         ctx->n_items = ctx->n_items_corner = ctx->n_big = ctx->n_stream = ctx->n_cluster = 0;
-        ctx->rows_robots.clear();
         ctx->cluster_groups.clear();
         VX_CK(ctx->d_plain_f.ensure(3 * (size_t)ctx->M_cap));
         VX_CK(cudaMemsetAsync(ctx->d_plain_f.p, 0, sizeof(float) * 3 * (size_t)ctx->M_cap, ctx->stream));
@@ -888,7 +884,6 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
     const bool damped = ctx->stepconst().damped != 0;
     std::vector<std::vector<std::pair<int, int>>> lattice(6), lattice_sp(6);
     std::vector<std::pair<int, std::pair<int, int>>> atomic;   // (threads, (-corners, robot))
-    std::vector<std::pair<int, int>> rows;                       // (-masses, robot), of the atomic ones
     std::vector<int> streamed;
     std::vector<std::pair<int, int>> clustered;                  // (q, robot)
     std::vector<int> mass_groups;                                // larger robots in mass-sized groups
@@ -966,10 +961,6 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
             // longest first: by spring count when known (a thread per spring), else corners
             const int key = (int)ctx->spring_count.size() == ctx->P ? ctx->spring_count[r] : C;
             atomic.push_back({threads, {-key, r}});
-            // no block size was asked for or tuned: the per-mass kernel where its rows fit (below)
-            if (ctx->p.accumulate == SIM_ACC_AUTO && ctx->p.threads <= 0 && ctx->class_threads[k] <= 0 && !damped &&
-                (int)ctx->mass_count.size() == ctx->P && rows_per_corner(C, budget) > 0)
-                rows.push_back({-ctx->mass_count[r], r});
         } else {
             streamed.push_back(r);
             ctx->max_stream_corner = std::max(ctx->max_stream_corner, C);
@@ -1023,27 +1014,6 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
         ctx->roles_max_corner = corners;
     }
     if (sim_status st = build_packed_items(ctx, lattice, mass_groups, damped)) return st;
-    // The per-mass kernel (step_rows.cu) takes every robot of the atomic kernel that it can, unless
-    // that would leave two launches that each fill only part of the SMs (20 robots 12x12x12 of 1884 to
-    // 2081 masses, split at 2048: 4.4 ms in two launches, 2.6 ms in one).  Undamped robots only:
-    // with dashpots its square roots cost more than the atomics they replace (100 robots 10x10x10,
-    // 200 steps: 2.17 ms on the atomic kernel, 2.44 on this one).
-    if (rows.size() < atomic.size() && (int)rows.size() < ctx->num_sms) rows.clear();
-    std::sort(rows.begin(), rows.end());               // longest first
-    ctx->rows_robots.clear();
-    ctx->rows_max_corner = 0;
-    ctx->rows_max_mass = rows.empty() ? 0 : -rows[0].first;
-    std::vector<char> in_rows(rows.empty() ? 0 : ctx->P, 0);
-    for (const auto& q : rows) {
-        ctx->rows_robots.push_back(q.second);
-        in_rows[q.second] = 1;
-        ctx->rows_max_corner = std::max(ctx->rows_max_corner, (int)(ctx->moff[q.second + 1] - ctx->moff[q.second]));
-    }
-    ctx->rows_nd = rows.empty() ? 0 : rows_per_corner(ctx->rows_max_corner, budget);
-    if (!rows.empty())
-        atomic.erase(std::remove_if(atomic.begin(), atomic.end(),
-                                    [&](const std::pair<int, std::pair<int, int>>& q) { return in_rows[q.second.second] != 0; }),
-                     atomic.end());
     std::sort(atomic.begin(), atomic.end());
     std::vector<int> big;
     for (size_t i = 0; i < atomic.size();) {
@@ -1079,8 +1049,8 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
         ctx->stream_cube40 = ctx->stream_cube40 && ctx->dims[3 * r] == 40 && ctx->dims[3 * r + 1] == 40 &&
                              ctx->dims[3 * r + 2] == 40;
     cudaStream_t s = ctx->stream;
-    VX_CK(ctx->d_queue.ensure(3 + ctx->atomic_groups.size()));
-    VX_CK(ctx->d_progress.ensure(std::max({items.size(), ctx->pitems.size(), ctx->rows_robots.size()})));
+    VX_CK(ctx->d_queue.ensure(2 + ctx->atomic_groups.size()));
+    VX_CK(ctx->d_progress.ensure(std::max(items.size(), ctx->pitems.size())));
     if (!streamed.empty()) {
         // both state buffers start equal (corners without a mass are never rewritten)
         VX_CK(ctx->d_x_alt.ensure(ctx->M_cap));
@@ -1091,7 +1061,7 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
     // all lists of the plan in one copy
     size_t total = 0;
     for (size_t bytes : {sizeof(int4) * items.size(), sizeof(int4) * ctx->pitems.size(), sizeof(int4) * ctx->pgroups.size(),
-                         sizeof(int) * robots.size(), sizeof(int) * big.size(), sizeof(int) * ctx->rows_robots.size(),
+                         sizeof(int) * robots.size(), sizeof(int) * big.size(),
                          sizeof(int) * cl_robots.size(), sizeof(int) * streamed.size()})
         total += Staging::padded(bytes);
     VX_CK(ctx->d_plan.ensure(total / sizeof(int4)));
@@ -1107,7 +1077,6 @@ static sim_status build_work_items(voxsim_ctx* ctx, const std::vector<int>* subs
         put(ctx->pgroups, ctx->d_pgroups);
         put(robots, ctx->d_item_robots);
         put(big, ctx->d_big);
-        put(ctx->rows_robots, ctx->d_rows);
         put(cl_robots, ctx->d_cluster);
         put(streamed, ctx->d_stream);
         VX_CK(cudaMemcpyAsync(ctx->d_plan.p, ctx->staging.p, total, cudaMemcpyHostToDevice, s));
@@ -1251,7 +1220,7 @@ static sim_status timing_pair(voxsim_ctx* ctx, cudaEvent_t ev[2])
     return SIM_OK;
 }
 
-// Segments per item of a persistent launch (lattice, packed lattice, force rows): with more items
+// Segments per item of a persistent launch (lattice, packed lattice): with more items
 // than SMs, each item's n steps are split, so that the last wave waits for one segment of the
 // slowest items instead of one whole run.  Among the splits with segments of at least kMinSegSteps
 // steps and at most kSegUnits units per SM, the one with the fewest step times on the busiest SM:
@@ -1259,8 +1228,7 @@ static sim_status timing_pair(voxsim_ctx* ctx, cudaEvent_t ev[2])
 // 5x5x5, 500 steps, take 1.62 ms in one (2 waves), 1.34 ms in 3 (5/3 waves) and 1.39 ms in 7 (12/7);
 // 600 robots 7x7x7 (3.95 waves), 500 steps, 3.80 ms in one and 3.88 ms in 7.
 // Against a fixed 64 units per SM of at least 256 steps from 512 steps on: 200 robots 6x9x5,
-// 500 steps, 2.18 -> 1.37 ms, 1000 robots 4x4x4 2.36 -> 1.35 ms, 500 robots 9x9x9 on the force rows
-// 3.42 -> 2.90 ms, 1024 robots 7x8x7 13.81 -> 13.69 ms, 1024 robots 8x8x8 (2000 steps) 29.27 ms both.
+// 500 steps, 2.18 -> 1.37 ms, 1000 robots 4x4x4 2.36 -> 1.35 ms, 1024 robots 7x8x7 13.81 -> 13.69 ms, 1024 robots 8x8x8 (2000 steps) 29.27 ms both.
 // A least segment of 24, 48 or 64 steps: within 1 %.
 constexpr int kMinSegSteps = 32, kSegUnits = 32, kSegSetupSteps = 2;
 static int lattice_segments(int items, int n, int sms)
@@ -1383,35 +1351,10 @@ static sim_status step_cluster(voxsim_ctx* ctx, int n)
     return SIM_OK;
 }
 
-// The robots of more than a block's corners and masses: the per-mass kernel of 1024-thread blocks,
-// and the atomic kernel, one persistent launch per thread count.
+// The atomic resident kernel: one persistent launch per thread count.
 static sim_status step_resident(voxsim_ctx* ctx, int n)
 {
     cudaStream_t s = ctx->stream;
-    if (!ctx->rows_robots.empty()) {
-        ResidentArgs a{};
-        a.pv = ctx->view();
-        a.corner_order = ctx->d_mass_corner.p;
-        a.cflags = ctx->d_cflags.p;
-        a.prm = ctx->d_prm.p;
-        a.x = ctx->d_x.p;
-        a.v = ctx->d_v.p;
-        a.sc = ctx->d_sc.p;
-        a.nsteps = n;
-        a.c = ctx->stepconst();
-        a.order = ctx->d_rows.p;
-        a.n_robots = (int)ctx->rows_robots.size();
-        a.queue = ctx->d_queue.p + 2 + ctx->atomic_groups.size();
-        a.max_mass = ctx->rows_max_corner;
-        a.nseg = lattice_segments(a.n_robots, n, ctx->num_sms);
-        a.seg_steps = (n + a.nseg - 1) / a.nseg;
-        a.progress = ctx->d_progress.p;
-        a.status = ctx->d_status.p + 2;
-        VX_CK(cudaMemsetAsync(a.progress, 0, sizeof(int) * a.n_robots, s));
-        VX_CK(cudaMemsetAsync(a.queue, 0, sizeof(int), s));
-        VX_LAUNCH(ctx, launch_step_rows(a, ctx->rows_nd, ctx->rows_max_mass, (size_t)ctx->smem_optin / 2 + 4096,
-                                        std::min(a.n_robots, ctx->num_sms), s));
-    }
     for (size_t gi = 0; gi < ctx->atomic_groups.size(); ++gi) {
         const voxsim_ctx::AtomicGroup& g = ctx->atomic_groups[gi];
         ResidentArgs a{};

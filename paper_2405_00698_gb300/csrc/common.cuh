@@ -168,21 +168,10 @@ struct ResidentArgs {
     int tm_rec;              // springs per thread held in tensor memory (0: none, nothing allocated)
     int tm_cols;             // tensor-memory columns per warp (of the block's 512)
     int accumulate;          // SIM_ACC_ATOMIC or SIM_ACC_GATHER
-    // step_rows.cu: the masses' corners (ascending), the parameter planes, and the segments of each
-    // robot's steps (as in LatticeArgs; nseg >= 1)
-    const int* corner_order;
-    const float* prm;
-    int nseg;
-    int seg_steps;
-    int* progress;
-    int* status;
 };
 cudaError_t launch_step_resident(const ResidentArgs& a, int grid, int threads, size_t smem,
                                  cudaStream_t s);
 
-// Robots with force rows in shared memory, undamped (step_rows.cu).
-int rows_per_corner(int corners, size_t budget);
-cudaError_t launch_step_rows(const ResidentArgs& a, int nd, int max_masses, size_t min_smem, int grid, cudaStream_t s);
 
 // Lattice-gather path (deterministic): work items of robots of one size class.
 struct LatticeArgs {
